@@ -238,7 +238,11 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * GEMM turns into digit planes itself, with the c E term moved to the right
  * operand ([E | X + cE].[B ; F] = [E | X].[B + cF ; F]), so that no digit
  * plane of the left operand goes through memory (for tall, narrow layers;
- * needs K words even for the 2-D loads) -- and
+ * needs K words even for the 2-D loads); or, tile_rows = 256, the residue path:
+ * products modulo 16 (Z_2^64) or 31 (Z_2^128) small moduli on 256-row tiles,
+ * put together by the Chinese remainder theorem (three kernels; odd N too; 2K
+ * up to 2^15; accepted for shapes near those the built-in rule gives it and for
+ * small ones) -- and
  * `swizzle` tiles per tile-order group (1-64); or path 0, the integer-pipe kernels, with tiles
  * of `tile_rows` rows (64 or 16; 0 = 16 when 64-row tiles would give fewer
  * blocks than SMs, else 64; skinny layers with M <= 8 use a GEMV whatever the
@@ -246,13 +250,19 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * shapes use a built-in rule (tensor cores from 2^22 ring MACs, 2^20 for
  * Z_2^128; the wide tile up to two of its row tiles, and for Z_2^128 up to
  * M = 64 when it has a work unit per SM; 64-row tiles up to M = 64, the tall tile for layers with N <= 64 and M >= 2048 (Z_2^64) or
- * M >= 1024 (Z_2^128), and for N <= 128 from M = 4096).  The table is process-wide and thread-safe; workspace
+ * M >= 1024 (Z_2^128), and for N <= 128 from M = 4096; and in place of the 128-row
+ * tiles and of the integer pipes the residue path wherever its estimated time is
+ * lower, which is for layers large in both output dimensions, from about 600 in
+ * Z_2^64 and 256 in Z_2^128, provided that the call's workspace covers it -- a
+ * smaller workspace that covers the other paths is accepted and gives the same
+ * result).  mpc_autotune_choice reports the tile that those other paths use for
+ * untuned shapes.  The table is process-wide and thread-safe; workspace
  * sizes do not depend on it.
  *
  * mpc_autotune: for each distinct shape of layers[count], times the
  *   candidates (128-row tiles, 64-row tiles for M <= 64, the wide tile for
  *   M <= 128, the tall tile for M >= 128, each with swizzle 1/4/8/16 on the
- *   tensor cores; tile heights 64 and 16 with K-split 1/2/4/8
+ *   tensor cores; the residue path; tile heights 64 and 16 with K-split 1/2/4/8
  *   on the integer pipes, below 2^31 ring MACs) on `stream` and stores the
  *   fastest.  Synchronous;
  *   allocates and frees its own scratch operands; do not call it during

@@ -511,7 +511,7 @@ def mpc_autotune(layers, stream=None) -> int:
 
 
 def mpc_autotune_set(layer, path: int, swizzle: int = 8, waves: int = 0, tile_rows: int = None):
-    """tile_rows: 128 or 64 for the tensor cores (default 128); 64, 16 or 0 (by grid size) for the
+    """tile_rows: 128, 64, 32 or 16 (wide), -128 (tall) or 256 (residue path) for the tensor cores (default 128); 64, 16 or 0 (by grid size) for the
     integer pipes (default 0)."""
     if tile_rows is None:
         tile_rows = 128 if path == 1 else 0

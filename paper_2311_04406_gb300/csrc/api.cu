@@ -57,12 +57,29 @@ int cuda_status(cudaError_t e) {
 // Workspace of a GEMM: the tensor-core digit planes whenever that kernel can
 // run the shape, so that any launch-table choice fits the same workspace.
 size_t gemm_ws(const mpc_layer* L, int one_half = 0) {
-    return mpcl::gemm_tc_workspace(L->M, L->K, L->N, L->ring.words, one_half);
+    size_t b = mpcl::gemm_tc_workspace(L->M, L->K, L->N, L->ring.words, one_half);
+    if (mpcl::gemm_crt_candidate(L->M, L->K, L->N, L->ring.words))
+        b = std::max(b, mpcl::gemm_crt_workspace(L->M, L->K, L->N, L->ring.words, one_half));
+    return b;
+}
+
+// 1 when the residue path runs the layer in this workspace, 0 when it does not
+// (no choice of it, or the built-in rule chose it and the workspace only covers
+// the other paths); negative status when the table demands it and it cannot.
+int use_crt(const mpcl::Choice& c, const mpcl::GemmArgs& g, const void* ws, size_t ws_bytes) {
+    if (!c.crt) return 0;
+    const bool fits = ws && ws_bytes >= mpcl::gemm_crt_workspace(g.M, g.K, g.N, g.words, g.one_half);
+    if (!fits) return c.tuned ? MPC_E_WORKSPACE : 0;
+    if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return MPC_E_ALIGN;
+    return 1;
 }
 
 int run_gemm(mpcl::GemmArgs g, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (g.M == 0 || g.N == 0) return MPC_OK;
     const mpcl::Choice c = mpcl::gemm_choice(g.M, g.K, g.N, g.words);
+    const int crt = use_crt(c, g, ws, ws_bytes);
+    if (crt < 0) return crt;
+    if (crt) return cuda_status(mpcl::launch_gemm_crt(g, ws, ws_bytes, st));
     if (c.path == 1) {
         if (!ws || ws_bytes < mpcl::gemm_tc_workspace(g.M, g.K, g.N, g.words, g.one_half))
             return MPC_E_WORKSPACE;
@@ -85,7 +102,8 @@ int mpc_version(void) { return 200; }
 int mpc_gemm_path(const mpc_layer* L) {
     int st = check_layer(L);
     if (st != MPC_OK) return st;
-    return mpcl::gemm_choice(L->M, L->K, L->N, L->ring.words).path;
+    const mpcl::Choice c = mpcl::gemm_choice(L->M, L->K, L->N, L->ring.words);
+    return c.crt ? 1 : c.path;
 }
 
 int mpc_launch_count(const mpc_layer* L, int which) {
@@ -99,6 +117,7 @@ int mpc_launch_count(const mpc_layer* L, int which) {
         case MPC_WS_PUBLIC_PRODUCT:
         case MPC_WS_TAG_FULL:
             if (M == 0 || N == 0) return 0;
+            if (mpcl::gemm_choice(M, K, N, w).crt) return mpcl::CRT_LAUNCHES;
             return mpcl::gemm_choice(M, K, N, w).path == 1 ? mpcl::gemm_tc_launches(M, K, N, w) : 1;
         case MPC_WS_TAG_COMPACT: return mpcl::compact_launches(M, K, N);
         case MPC_WS_CHECK_COMPACT: return 1;
@@ -411,7 +430,18 @@ bool on_tc(const mpc_layer& L) {
 }
 
 // workspace of a grouped GEMM: the digit planes of every layer the
-// tensor-core kernel can run (whatever the launch table picks)
+// tensor-core kernel can run (whatever the launch table picks), then one
+// region that the layers of the residue path take in turn
+size_t group_crt_ws(const mpc_layer* layers, int count) {
+    size_t t = 0;
+    for (int i = 0; i < count; ++i) {
+        const mpc_layer& L = layers[i];
+        if (L.M > 0 && L.N > 0 && mpcl::gemm_crt_candidate(L.M, L.K, L.N, L.ring.words))
+            t = std::max(t, mpcl::gemm_crt_workspace(L.M, L.K, L.N, L.ring.words));
+    }
+    return t;
+}
+
 size_t group_gemm_ws(const mpc_layer* layers, int count) {
     size_t t = 0;
     for (int i = 0; i < count; ++i)
@@ -476,14 +506,22 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
         if (!ws || ws_bytes < need) return MPC_E_WORKSPACE;
         if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return MPC_E_ALIGN;
     }
-    std::vector<mpcl::GemmArgs> tc, simt;
+    // the residue path's region follows the digit planes; a workspace without it
+    // is accepted as long as no table entry demands that path
+    std::vector<mpcl::GemmArgs> tc, simt, crt;
+    uint8_t* crt_ws = ws ? static_cast<uint8_t*>(ws) + need : nullptr;
+    const size_t crt_bytes = ws_bytes > need ? ws_bytes - need : 0;
     std::vector<uint8_t*> ap;
     uint8_t* cur = static_cast<uint8_t*>(ws);
     for (int i = 0; i < count; ++i) {
         if (g[i].M == 0 || g[i].N == 0) continue;
         const mpcl::Choice c = mpcl::gemm_choice(g[i].M, g[i].K, g[i].N, g[i].words);
         mpcl::GemmArgs x = g[i];
-        if (c.path == 1) {
+        const int use = use_crt(c, x, crt_ws, crt_bytes);
+        if (use < 0) return use;
+        if (use) {
+            crt.push_back(x);
+        } else if (c.path == 1) {
             x.gm = c.gm;
             x.rows = c.rows;
             tc.push_back(x);
@@ -495,9 +533,15 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
         }
         cur += (mpcl::gemm_tc_workspace(g[i].M, g[i].K, g[i].N, g[i].words) + 255) & ~size_t(255);
     }
-    SidePool* side = (!simt.empty() && simt.size() + (tc.empty() ? 0 : 1) >= 2) ? side_pool() : nullptr;
+    auto run_crt = [&]() -> int {
+        for (const auto& x : crt) CHK(cuda_status(mpcl::launch_gemm_crt(x, crt_ws, crt_bytes, st)));
+        return MPC_OK;
+    };
+    const bool tensor = !tc.empty() || !crt.empty();
+    SidePool* side = (!simt.empty() && simt.size() + (tensor ? 1 : 0) >= 2) ? side_pool() : nullptr;
     if (!side) {
         if (!tc.empty()) CHK(cuda_status(mpcl::launch_gemm_tc_grouped(tc.data(), (int)tc.size(), ap.data(), st)));
+        CHK(run_crt());
         for (const auto& x : simt) CHK(cuda_status(mpcl::launch_gemm_simt(x, st)));
         return MPC_OK;
     }
@@ -513,6 +557,7 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
         status = cuda_status(mpcl::launch_gemm_simt(simt[j], side->s[j % ns]));
     if (status == MPC_OK && !tc.empty())
         status = cuda_status(mpcl::launch_gemm_tc_grouped(tc.data(), (int)tc.size(), ap.data(), st));
+    if (status == MPC_OK) status = run_crt();
     for (int i = 0; i < ns; ++i) {
         const int a = cuda_status(cudaEventRecord(side->join[i], side->s[i]));
         const int b = a == MPC_OK ? cuda_status(cudaStreamWaitEvent(st, side->join[i], 0)) : a;
@@ -605,7 +650,7 @@ size_t mpc_workspace_size_grouped(const mpc_layer* layers, int count, int which)
     }
     switch (which) {
         case MPC_WS_SHARE:
-        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count);
+        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count) + group_crt_ws(layers, count);
         case MPC_WS_TAG_COMPACT: return group_compact_ws(layers, count);
         default: return 0;
     }
@@ -622,7 +667,9 @@ int mpc_launch_count_grouped(const mpc_layer* layers, int count, int which) {
         if (!same_ring(layers[i].ring, layers[0].ring)) return MPC_E_RING;
         const mpc_layer& L = layers[i];
         if (which == MPC_WS_SHARE || which == MPC_WS_TAG_FULL) {
-            if (on_tc(L)) {
+            if (L.M > 0 && L.N > 0 && mpcl::gemm_choice(L.M, L.K, L.N, L.ring.words).crt) {
+                n += mpcl::CRT_LAUNCHES;
+            } else if (on_tc(L)) {
                 tM.push_back(L.M);
                 tK.push_back(L.K);
                 tN.push_back(L.N);

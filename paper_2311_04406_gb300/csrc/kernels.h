@@ -45,12 +45,15 @@ struct Choice {
     int waves;
     int tuned;
     int rows;
+    int crt;    // the residue path runs the layer when the workspace holds it
 };
 Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words);
 int wide_tile_rows(int words);   // the launch-table value of the wide tensor-core tile
 // the launch-table value of the tall tensor-core tile (128-row tiles whose
 // left operand the GEMM converts itself)
 constexpr int TALL_TILE_ROWS = -128;
+// the launch-table value of the residue path (gemm_crt.cu: 256 x 256 tiles)
+constexpr int CRT_TILE_ROWS = 256;
 
 cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t st);
 
@@ -70,7 +73,19 @@ bool gemm_tc_eligible(int64_t M, int64_t K, int64_t N, int words);   // heuristi
 // the kernel can run the shape with `rows`-row tiles (128 or 64)
 bool gemm_tc_feasible(int64_t M, int64_t K, int64_t N, int words, int rows = 128);
 int gemm_tc_launches(int64_t M, int64_t K, int64_t N, int words);
+void* tensor_map_encoder();       // the driver's cuTensorMapEncodeTiled, or NULL
 int tc_timeout_flag(bool* set);   // synchronous; 0 on success
+
+// ring GEMM from residue products (exact); layers large in both output
+// dimensions.  A candidate is a shape whose workspace covers this path, a
+// superset of the shapes the built-in rule runs on it.
+bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
+bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words);
+bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words);
+size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
+constexpr int CRT_LAUNCHES = 3;
+cudaError_t launch_gemm_crt(const GemmArgs& a, void* ws, size_t ws_bytes, cudaStream_t st);
+int crt_timeout_flag(bool* set, cudaStream_t s);   // synchronous; 0 on success
 
 // CompactTag path (a3, a4, a5)
 struct CompactArgs {

@@ -5,7 +5,7 @@
 // (ring width, M, K, N) the table holds a Choice: the tensor-core kernel with
 // a tile height (128 or 64 rows) and a row-tile swizzle width, or the
 // integer-pipe kernels with a tile height (64 or 16 rows; 0 = by grid size)
-// and a K-split target.  Shapes not in the table use
+// and a K-split target, or the residue path (gemm_crt.cu, tile height 256).  Shapes not in the table use
 // the built-in heuristic (gemm_tc_eligible; 64-row tiles for M <= 64).
 // mpc_autotune times the candidates of each distinct shape on the caller's
 // stream and stores the fastest; the table can be saved to and loaded from a
@@ -14,6 +14,7 @@
 //     <words> <M> <K> <N> <path> <rows> <swizzle> <waves>   (one line per shape)
 // (version 1 files, without <rows>, load as 128-row tiles).  The table is
 // process-wide and guarded by a mutex.
+#include <algorithm>
 #include <cstdio>
 #include <map>
 #include <mutex>
@@ -39,6 +40,8 @@ std::map<Key, Choice>& table() {
 }
 
 bool choice_ok(const Choice& c, int64_t M, int64_t K, int64_t N, int words) {
+    if (c.path == 1 && c.rows == CRT_TILE_ROWS)
+        return gemm_crt_candidate(M, K, N, words) && c.gm >= 1 && c.gm <= 64;
     if (c.path == 1)
         return (c.rows == 64 || c.rows == 128 || c.rows == wide_tile_rows(words) || c.rows == TALL_TILE_ROWS) &&
                gemm_tc_feasible(M, K, N, words, c.rows) && c.gm >= 1 && c.gm <= 64;
@@ -80,7 +83,11 @@ Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words) {
     {
         std::lock_guard<std::mutex> lk(g_mu);
         auto it = table().find(Key{words, M, K, N});
-        if (it != table().end()) return it->second;
+        if (it != table().end()) {
+            Choice c = it->second;
+            c.crt = c.path == 1 && c.rows == CRT_TILE_ROWS;
+            return c;
+        }
     }
     Choice c;
     c.path = gemm_tc_eligible(M, K, N, words) ? 1 : 0;
@@ -88,6 +95,7 @@ Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words) {
     c.waves = 0;
     c.tuned = 0;
     c.rows = c.path == 1 ? default_rows(M, K, N, words) : 0;
+    c.crt = gemm_crt_preferred(M, K, N, words) ? 1 : 0;
     return c;
 }
 
@@ -111,6 +119,7 @@ float time_candidate(const mpcl::GemmArgs& a, const mpcl::Choice& c, void* ws, s
     g.simt_waves = c.waves;
     g.rows = c.rows;
     auto run = [&]() -> cudaError_t {
+        if (c.path == 1 && c.rows == mpcl::CRT_TILE_ROWS) return mpcl::launch_gemm_crt(g, ws, ws_bytes, st);
         return c.path == 1 ? mpcl::launch_gemm_tc(g, ws, ws_bytes, st) : mpcl::launch_gemm_simt(g, st);
     };
     *ok = false;
@@ -167,6 +176,8 @@ int mpc_autotune(const mpc_layer* layers, int count, void* stream) {
                 if (!mpcl::gemm_tc_feasible(M, K, N, w, rows)) continue;
                 for (int gm : {1, 4, 8, 16}) cands.push_back(mpcl::Choice{1, gm, 0, 1, rows});
             }
+        const bool crt = mpcl::gemm_crt_candidate(M, K, N, w);
+        if (crt) cands.push_back(mpcl::Choice{1, 1, 0, 1, mpcl::CRT_TILE_ROWS, 1});
         // the integer pipes are far slower on large products: not timed there;
         // their tile height (64 or 16 rows) matters only above M = 8
         if (!tc || macs < 2147483648.0)
@@ -177,7 +188,8 @@ int mpc_autotune(const mpc_layer* layers, int count, void* stream) {
         // operands (contents do not matter for the time: every path is exact)
         const size_t e = 8 * (size_t)w;
         const size_t b_mk = e * (size_t)(M * K), b_kn = e * (size_t)(K * N), b_mn = e * (size_t)(M * N);
-        const size_t ws_bytes = tc ? mpcl::gemm_tc_workspace(M, K, N, w) : 0;
+        size_t ws_bytes = tc ? mpcl::gemm_tc_workspace(M, K, N, w) : 0;
+        if (crt) ws_bytes = std::max(ws_bytes, mpcl::gemm_crt_workspace(M, K, N, w));
         void *E = nullptr, *X = nullptr, *B = nullptr, *F = nullptr, *C = nullptr, *Z = nullptr, *ws = nullptr;
         bool alloc = cudaMalloc(&E, b_mk > 0 ? b_mk : 16) == cudaSuccess &&
                      cudaMalloc(&X, b_mk > 0 ? b_mk : 16) == cudaSuccess &&
