@@ -429,25 +429,27 @@ bool on_tc(const mpc_layer& L) {
     return L.M > 0 && L.N > 0 && mpcl::gemm_choice(L.M, L.K, L.N, L.ring.words).path == 1;
 }
 
-// workspace of a grouped GEMM: the digit planes of every layer the
-// tensor-core kernel can run (whatever the launch table picks), then one
-// region that the layers of the residue path take in turn
-size_t group_crt_ws(const mpc_layer* layers, int count) {
-    size_t t = 0;
-    for (int i = 0; i < count; ++i) {
-        const mpc_layer& L = layers[i];
-        if (L.M > 0 && L.N > 0 && mpcl::gemm_crt_candidate(L.M, L.K, L.N, L.ring.words))
-            t = std::max(t, mpcl::gemm_crt_workspace(L.M, L.K, L.N, L.ring.words));
-    }
-    return t;
+// Workspace of a grouped GEMM: one region per layer, each as large as the layer's
+// own call needs (whatever the launch table picks); without the residue path,
+// the digit planes alone.
+size_t region(const mpc_layer& L, bool with_crt) {
+    if (L.M == 0 || L.N == 0) return 0;
+    const size_t b = with_crt ? gemm_ws(&L) : mpcl::gemm_tc_workspace(L.M, L.K, L.N, L.ring.words);
+    return (b + 255) & ~size_t(255);
 }
 
-size_t group_gemm_ws(const mpc_layer* layers, int count) {
+// In a group, Z_2^64 layers that the digit tiles can run stay with them unless
+// the table says otherwise: they share one launch pair with the group's other
+// layers, where a layer on the residue path runs by itself (48 uneven layers:
+// 1427 us per step with the digits, 1421 us with the rule's three layers on the
+// residue path).
+bool group_uses_crt(const mpcl::Choice& c, int64_t M, int64_t K, int64_t N, int words) {
+    return c.crt && (c.tuned || words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words));
+}
+
+size_t group_gemm_ws(const mpc_layer* layers, int count, bool with_crt) {
     size_t t = 0;
-    for (int i = 0; i < count; ++i)
-        if (layers[i].M > 0 && layers[i].N > 0)
-            t += (mpcl::gemm_tc_workspace(layers[i].M, layers[i].K, layers[i].N, layers[i].ring.words) + 255) &
-                 ~size_t(255);
+    for (int i = 0; i < count; ++i) t += region(layers[i], with_crt);
     return t;
 }
 
@@ -501,26 +503,27 @@ SidePool* side_pool() {
 
 int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, void* ws, size_t ws_bytes,
                    cudaStream_t st) {
-    const size_t need = group_gemm_ws(layers, count);
+    // a workspace without the residue path's planes is accepted as long as no
+    // table entry demands that path
+    const bool with_crt = ws_bytes >= group_gemm_ws(layers, count, true);
+    const size_t need = group_gemm_ws(layers, count, with_crt);
     if (need > 0) {
         if (!ws || ws_bytes < need) return MPC_E_WORKSPACE;
         if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return MPC_E_ALIGN;
     }
-    // the residue path's region follows the digit planes; a workspace without it
-    // is accepted as long as no table entry demands that path
     std::vector<mpcl::GemmArgs> tc, simt, crt;
-    uint8_t* crt_ws = ws ? static_cast<uint8_t*>(ws) + need : nullptr;
-    const size_t crt_bytes = ws_bytes > need ? ws_bytes - need : 0;
-    std::vector<uint8_t*> ap;
+    std::vector<uint8_t*> ap, cp;
     uint8_t* cur = static_cast<uint8_t*>(ws);
     for (int i = 0; i < count; ++i) {
         if (g[i].M == 0 || g[i].N == 0) continue;
         const mpcl::Choice c = mpcl::gemm_choice(g[i].M, g[i].K, g[i].N, g[i].words);
         mpcl::GemmArgs x = g[i];
-        const int use = use_crt(c, x, crt_ws, crt_bytes);
+        const size_t bytes = region(layers[i], with_crt);
+        const int use = group_uses_crt(c, x.M, x.K, x.N, x.words) ? use_crt(c, x, with_crt ? cur : nullptr, bytes) : 0;
         if (use < 0) return use;
         if (use) {
             crt.push_back(x);
+            cp.push_back(cur);
         } else if (c.path == 1) {
             x.gm = c.gm;
             x.rows = c.rows;
@@ -531,10 +534,12 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
             x.rows = c.rows;
             simt.push_back(x);
         }
-        cur += (mpcl::gemm_tc_workspace(g[i].M, g[i].K, g[i].N, g[i].words) + 255) & ~size_t(255);
+        cur += bytes;
     }
     auto run_crt = [&]() -> int {
-        for (const auto& x : crt) CHK(cuda_status(mpcl::launch_gemm_crt(x, crt_ws, crt_bytes, st)));
+        for (size_t j = 0; j < crt.size(); ++j)
+            CHK(cuda_status(mpcl::launch_gemm_crt(
+                crt[j], cp[j], mpcl::gemm_crt_workspace(crt[j].M, crt[j].K, crt[j].N, crt[j].words), st)));
         return MPC_OK;
     };
     const bool tensor = !tc.empty() || !crt.empty();
@@ -650,7 +655,7 @@ size_t mpc_workspace_size_grouped(const mpc_layer* layers, int count, int which)
     }
     switch (which) {
         case MPC_WS_SHARE:
-        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count) + group_crt_ws(layers, count);
+        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count, true);
         case MPC_WS_TAG_COMPACT: return group_compact_ws(layers, count);
         default: return 0;
     }
@@ -667,7 +672,8 @@ int mpc_launch_count_grouped(const mpc_layer* layers, int count, int which) {
         if (!same_ring(layers[i].ring, layers[0].ring)) return MPC_E_RING;
         const mpc_layer& L = layers[i];
         if (which == MPC_WS_SHARE || which == MPC_WS_TAG_FULL) {
-            if (L.M > 0 && L.N > 0 && mpcl::gemm_choice(L.M, L.K, L.N, L.ring.words).crt) {
+            if (L.M > 0 && L.N > 0 &&
+                group_uses_crt(mpcl::gemm_choice(L.M, L.K, L.N, L.ring.words), L.M, L.K, L.N, L.ring.words)) {
                 n += mpcl::CRT_LAUNCHES;
             } else if (on_tc(L)) {
                 tM.push_back(L.M);

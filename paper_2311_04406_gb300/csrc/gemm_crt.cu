@@ -1071,7 +1071,7 @@ double crt_ratio(int64_t M, int64_t K, int64_t N, int words) {
 // launch table may then demand the path).
 bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words) {
     const double r = crt_ratio(M, K, N, words);
-    return r < 1.3 || (r < 1e9 && crt_plan(M, K, N, words, 0).total <= (size_t(32) << 20));
+    return r < 1.1 || (r < 1e9 && crt_plan(M, K, N, words, 0).total <= (size_t(32) << 20));
 }
 bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words) { return crt_ratio(M, K, N, words) < 0.95; }
 
