@@ -1,8 +1,10 @@
-"""Thin ctypes binding of the C ABI in include/mpclinear.h.
+"""Thin binding of the C ABI in include/mpclinear.h.
 
 Argument marshalling only: torch tensors supply device pointers and the
 current CUDA stream; every step of the computation runs in the library's
-kernels.  Each function has the C name and raises `MpcError` on a non-zero
+kernels.  The calls that run per layer marshal their arguments in native code
+(csrc/binding.c); ctypes is the general path, which every call that fails a
+check there takes, and which raises.  Each function has the C name and raises `MpcError` on a non-zero
 status.  If the shared library is missing, loading raises immediately: there
 is no fallback path.
 
@@ -19,6 +21,7 @@ from . import build as _build
 
 _lock = threading.Lock()
 _lib = None
+_nat = None          # the native marshalling, loaded with the library
 
 MPC_TAG_FULL, MPC_TAG_COMPACT, MPC_TAG_COMPACT_TRUNC = 0, 1, 2
 MPC_CHECK_COMPACT, MPC_CHECK_BATCHREC, MPC_CHECK_BATCHREC_SEEDED = 0, 1, 2
@@ -161,6 +164,12 @@ def load(build_if_missing: bool = False):
         lib.mpc_gemm_path.restype = ctypes.c_int
         lib.mpc_version.argtypes = []
         lib.mpc_version.restype = ctypes.c_int
+        if not os.path.exists(_build.BINDING):
+            raise RuntimeError(f"{_build.BINDING} is not built; run `python -c 'import __graft_entry__ as g; g.build()'`")
+        from . import _binding
+        _binding.open(path)
+        global _nat
+        _nat = _binding
         _lib = lib
         return lib
 
@@ -215,13 +224,43 @@ def _args(fn, layer, elems, given):
     return [_sized(fn, n, t, elems[n], w) if n in elems else _ptr(t) for n, t in given.items()]
 
 
+_raw_stream = None
+
+
+def _current_stream():
+    """Handle of the current stream of the current device (torch's Python-level
+    stream object costs several microseconds per call)."""
+    global _raw_stream
+    import torch
+    if _raw_stream is None:
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+            (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+def _native(fn, name, stream, *args, ws=0, alloc=None):
+    """Status of the native call `name` (raised when it is an error), or None
+    when the general path has to handle the arguments.  ws: a workspace tensor
+    or address, None to allocate one with alloc(), 0 for calls without one."""
+    if _nat is None:
+        load()
+    try:
+        s = _stream(stream)
+        w = () if alloc is None else (ws, -1) if ws is not None else alloc()
+    except (RuntimeError, AssertionError):
+        return None          # no CUDA device: the general path checks the arguments first
+    r = getattr(_nat, name)(*args, *w, s)
+    if r:
+        _check(fn, r)
+    return r
 
 
 def _check(fn: str, status: int):
@@ -283,6 +322,9 @@ def _alloc_ws(need, stream):
 
 
 def mpc_linear_share(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None):
+    if _native("mpc_linear_share", "share", stream, layer, E, F, A_i, B_i, C_i, Z_i, ws=ws,
+               alloc=lambda: _ws(layer, MPC_WS_SHARE, None, stream)) is not None:
+        return Z_i
     a = _args("mpc_linear_share", layer, _share_elems(layer.M, layer.K, layer.N),
               dict(E=E, F=F, A_i=A_i, B_i=B_i, C_i=C_i, Z_i=Z_i))
     wp, wb = _ws(layer, MPC_WS_SHARE, ws, stream)
@@ -293,6 +335,9 @@ def mpc_linear_share(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None):
 def mpc_linear_tag(layer, mode, alpha_i, E, F, mA_i, mB_i, mC_i, mZ_i, mR_i=None, Dtilde=None,
                    chi=None, mDc_i=None, Dc=None, ws=None, stream=None):
     which = MPC_WS_TAG_FULL if mode == MPC_TAG_FULL else MPC_WS_TAG_COMPACT
+    if _native("mpc_linear_tag", "tag", stream, layer, mode, alpha_i, E, F, mA_i, mB_i, mC_i, mR_i, Dtilde, chi, mZ_i,
+               mDc_i, Dc, ws=ws, alloc=lambda: _ws(layer, which, None, stream)) is not None:
+        return mZ_i
     a = _args("mpc_linear_tag", layer, _tag_elems(layer.M, layer.K, layer.N, mode),
               dict(alpha_i=alpha_i, E=E, F=F, mA_i=mA_i, mB_i=mB_i, mC_i=mC_i, mR_i=mR_i, Dtilde=Dtilde,
                    chi=chi, mZ_i=mZ_i, mDc_i=mDc_i, Dc=Dc))
@@ -304,6 +349,9 @@ def mpc_linear_tag(layer, mode, alpha_i, E, F, mA_i, mB_i, mC_i, mZ_i, mR_i=None
 
 def mpc_tag_check(layer, mode, alpha_i, chi_hat, opened, tag_i, cs_i, ws=None, stream=None):
     which = MPC_WS_CHECK_COMPACT if mode == MPC_CHECK_COMPACT else MPC_WS_CHECK_BATCHREC
+    if _native("mpc_tag_check", "check", stream, layer, mode, alpha_i, chi_hat, opened, tag_i, cs_i, ws=ws,
+               alloc=lambda: _ws(layer, which, None, stream)) is not None:
+        return cs_i
     fn, w = "mpc_tag_check", layer.ring.words
     n = layer.M if mode == MPC_CHECK_COMPACT else layer.M * layer.N
     # the seeded BATCHREC check reads one 64-bit seed word, not ring elements
@@ -330,6 +378,9 @@ def mpc_linear_tag_compact_noalloc(layer, alpha_i, E, F, mA_i, mB_i, mC_i, mR_i,
 
 def mpc_linear_share_trunc(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None):
     """Truncated layer, step 2: Z_i = C_i + E.B_i + A_i.F for every party."""
+    if _native("mpc_linear_share_trunc", "share_trunc", stream, layer, E, F, A_i, B_i, C_i, Z_i, ws=ws,
+               alloc=lambda: _ws(layer, MPC_WS_SHARE_TRUNC, None, stream)) is not None:
+        return Z_i
     a = _args("mpc_linear_share_trunc", layer, _share_elems(layer.M, layer.K, layer.N),
               dict(E=E, F=F, A_i=A_i, B_i=B_i, C_i=C_i, Z_i=Z_i))
     wp, wb = _ws(layer, MPC_WS_SHARE_TRUNC, ws, stream)
@@ -340,6 +391,9 @@ def mpc_linear_share_trunc(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None
 
 def mpc_public_product(layer, E, F, P, ws=None, stream=None):
     """P = E.F (public)."""
+    if _native("mpc_public_product", "public_product", stream, layer, E, F, P, ws=ws,
+               alloc=lambda: _ws(layer, MPC_WS_PUBLIC_PRODUCT, None, stream)) is not None:
+        return P
     M, K, N = layer.M, layer.K, layer.N
     a = _args("mpc_public_product", layer, dict(E=M * K, F=K * N, P=M * N), dict(E=E, F=F, P=P))
     wp, wb = _ws(layer, MPC_WS_PUBLIC_PRODUCT, ws, stream)
@@ -349,6 +403,9 @@ def mpc_public_product(layer, E, F, P, ws=None, stream=None):
 
 def mpc_optmac_trunc(layer, f, alpha_i, Rf_i, mRf_i, Dtilde, P, Zf_i, mZf_i, stream=None):
     """Truncated layer, steps 3-4 (OptMAC&Trunc plus the public product term)."""
+    if _native("mpc_optmac_trunc", "optmac_trunc", stream, layer, f, alpha_i, Rf_i, mRf_i, Dtilde, P, Zf_i,
+               mZf_i) is not None:
+        return Zf_i, mZf_i
     MN = layer.M * layer.N
     a = _args("mpc_optmac_trunc", layer, dict(alpha_i=1, Rf_i=MN, mRf_i=MN, Dtilde=MN, P=MN, Zf_i=MN, mZf_i=MN),
               dict(alpha_i=alpha_i, Rf_i=Rf_i, mRf_i=mRf_i, Dtilde=Dtilde, P=P, Zf_i=Zf_i, mZf_i=mZf_i))
@@ -358,6 +415,9 @@ def mpc_optmac_trunc(layer, f, alpha_i, Rf_i, mRf_i, Dtilde, P, Zf_i, mZf_i, str
 
 def mpc_batchrec_mask(k, s, rows, cols, X_i, A_i, R_i, mX_i, mA_i, mR_i, W_i, mW_i, stream=None):
     """Pi_BatchRec open phase step 1: W_i = X_i - A_i + R_i and the same for the tags."""
+    if _native("mpc_batchrec_mask", "batchrec_mask", stream, k, s, rows, cols, X_i, A_i, R_i, mX_i, mA_i, mR_i, W_i,
+               mW_i) is not None:
+        return W_i, mW_i
     ring = mpc_ring(int(k), int(s), (int(k) + int(s) + 63) // 64)
     fn, n = "mpc_batchrec_mask", int(rows) * int(cols)
     a = [_sized(fn, name, t, n, ring.words) for name, t in
@@ -369,6 +429,8 @@ def mpc_batchrec_mask(k, s, rows, cols, X_i, A_i, R_i, mX_i, mA_i, mR_i, W_i, mW
 
 def mpc_lincomb(k, s, coefs, ins, out, stream=None):
     """out = sum_j coefs[j] * ins[j] (elementwise, mod 2^(k+s)); ins are tensors of out's shape."""
+    if _native("mpc_lincomb", "lincomb", stream, k, s, coefs, ins, out) is not None:
+        return out
     ring = mpc_ring(int(k), int(s), (int(k) + int(s) + 63) // 64)
     n = out.numel() // ring.words if out is not None and hasattr(out, "numel") else 0
     c = (ctypes.c_int64 * len(coefs))(*[int(x) for x in coefs])
@@ -383,6 +445,8 @@ def mpc_lincomb_grouped(k, s, coefs, ins, outs, stream=None, n=None):
     """outs[g] = sum_j coefs[j] * ins[g][j] for every group g (one launch per 64 groups).
     n[g]: ring elements of group g; taken from outs[g] when omitted (tensors),
     required when the buffers are raw addresses."""
+    if _native("mpc_lincomb_grouped", "lincomb_grouped", stream, k, s, coefs, ins, outs, n) is not None:
+        return outs
     ring = mpc_ring(int(k), int(s), (int(k) + int(s) + 63) // 64)
     G = len(outs)
     if G == 0:
@@ -404,6 +468,8 @@ def mpc_tag_check_grouped(layers, ptrs, stream=None):
     """Compact check shares of many layers: ptrs[i] is a dict of CHECK_PTR_FIELDS tensors."""
     if not layers:
         return
+    if _native("mpc_tag_check_grouped", "check_grouped", stream, layers, ptrs) is not None:
+        return
     arr = (mpc_layer * len(layers))(*layers)
     pa = (mpc_check_ptrs * len(layers))()
     for i, d in enumerate(ptrs):
@@ -416,6 +482,9 @@ def mpc_tag_check_grouped(layers, ptrs, stream=None):
 
 def mpc_im2col(k, s, batch, channels, height, width, f, pad, stride, src, dst, stream=None):
     """dst = the im2col matrix of NCHW images src for an f x f filter (zero padding, stride)."""
+    if _native("mpc_im2col", "im2col", stream, k, s, batch, channels, height, width, f, pad, stride, src,
+               dst) is not None:
+        return dst
     ring = mpc_ring(int(k), int(s), (int(k) + int(s) + 63) // 64)
     src_p, dst_p = _ptr(src), _ptr(dst)
     if f >= 1 and 0 <= pad < f and stride >= 1 and height + 2 * pad >= f and width + 2 * pad >= f:
@@ -430,6 +499,8 @@ def mpc_im2col(k, s, batch, channels, height, width, f, pad, stride, src, dst, s
 
 def mpc_transpose(k, s, rows, cols, src, dst, stream=None):
     """dst (cols x rows) = src (rows x cols)^T, ring elements of Z_2^(k+s)."""
+    if _native("mpc_transpose", "transpose", stream, k, s, rows, cols, src, dst) is not None:
+        return dst
     ring = mpc_ring(int(k), int(s), (int(k) + int(s) + 63) // 64)
     n = int(rows) * int(cols)
     _check("mpc_transpose", load().mpc_transpose(ctypes.byref(ring), int(rows), int(cols),
@@ -482,6 +553,9 @@ def _ws_grouped(layers, which, ws, stream=None):
 def mpc_linear_share_grouped(layers, ptrs, ws=None, stream=None):
     """Shares of many layers in one call (same results as one mpc_linear_share per layer)."""
     fn = "mpc_linear_share_grouped"
+    if _native(fn, "share_grouped", stream, layers, ptrs, ws=ws,
+               alloc=lambda: _ws_grouped(layers, MPC_WS_SHARE, None, stream)) is not None:
+        return
     pa = _ptr_array(mpc_share_ptrs, SHARE_PTR_FIELDS, ptrs, fn, layers, lambda L: _share_elems(L.M, L.K, L.N))
     wp, wb = _ws_grouped(layers, MPC_WS_SHARE, ws, stream)
     _check(fn, load().mpc_linear_share_grouped(_layer_array(layers), len(layers), pa, wp, wb, _stream(stream)))
@@ -491,6 +565,9 @@ def mpc_linear_tag_grouped(layers, mode, ptrs, ws=None, stream=None):
     """Tags of many layers in one call (same results as one mpc_linear_tag per layer)."""
     which = MPC_WS_TAG_FULL if mode == MPC_TAG_FULL else MPC_WS_TAG_COMPACT
     fn = "mpc_linear_tag_grouped"
+    if _native(fn, "tag_grouped", stream, layers, mode, ptrs, ws=ws,
+               alloc=lambda: _ws_grouped(layers, which, None, stream)) is not None:
+        return
     pa = _ptr_array(mpc_tag_ptrs, TAG_PTR_FIELDS, ptrs, fn, layers, lambda L: _tag_elems(L.M, L.K, L.N, mode))
     wp, wb = _ws_grouped(layers, which, ws, stream)
     _check(fn, load().mpc_linear_tag_grouped(_layer_array(layers), len(layers), int(mode), pa, wp, wb,

@@ -1,4 +1,5 @@
-"""Build libmpclinear.so in-tree with nvcc for sm_103a (GB300).
+"""Build libmpclinear.so in-tree with nvcc for sm_103a (GB300), and _binding.so,
+the native argument marshalling of abi.py, with the host compiler.
 
 Each .cu file is compiled to an object in parallel, then linked into one
 shared library with the CUDA runtime linked statically.  The build is skipped
@@ -11,6 +12,8 @@ import hashlib
 import os
 import shutil
 import subprocess
+import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -18,6 +21,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libmpclinear.so")
+BINDING = os.path.join(HERE, "_binding.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
@@ -37,13 +41,13 @@ def _sources():
 
 def _digest(extra=()) -> str:
     h = hashlib.sha256()
-    files = _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + \
+    files = _sources() + [os.path.join(CSRC, "binding.c")] + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + \
         sorted(glob.glob(os.path.join(CSRC, "*.h"))) + [os.path.join(ROOT, "include", "mpclinear.h")]
     for f in files:
         h.update(f.encode())
         with open(f, "rb") as fh:
             h.update(fh.read())
-    h.update(" ".join(ARCH + FLAGS + list(extra)).encode())
+    h.update(" ".join(ARCH + FLAGS + list(extra) + [sys.version]).encode())
     return h.hexdigest()
 
 
@@ -52,7 +56,8 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(BUILD, exist_ok=True)
     stamp = os.path.join(BUILD, "libmpclinear.sha256")
     dig = _digest(extra_flags)
-    if not force and os.path.exists(LIB) and os.path.exists(stamp) and open(stamp).read() == dig:
+    if not force and os.path.exists(LIB) and os.path.exists(BINDING) and os.path.exists(stamp) and \
+             open(stamp).read() == dig:
         return LIB
 
     def compile_one(src):
@@ -74,6 +79,16 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if not cc:
+        raise RuntimeError("a C compiler is required to build the binding")
+    tmp = BINDING + f".{os.getpid()}.tmp"
+    r = subprocess.run([cc, "-O2", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"),
+                        "-I" + sysconfig.get_paths()["include"], "-o", tmp, os.path.join(CSRC, "binding.c"), "-ldl"],
+                       capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"the binding does not compile:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
     with open(stamp, "w") as fh:
         fh.write(dig)
     return LIB
