@@ -5,14 +5,14 @@
 //   a5  mZc  = mC.chi + E.(mB.chi) + mA.(F.chi) + alpha * E.(F.chi)
 //       mDc  = mR.chi - mZc,  Dc = D~.chi            (Eq. (compute-zcomptag))
 //
-// In Z_2^64 the two terms in E are one product: E.(mB.chi) + alpha * E.(F.chi)
-// = E.(mB.chi + alpha * F.chi) mod 2^64 (the ring is commutative and the sums
-// distribute).  The rows pass stores w = mB.chi + alpha * F.chi in place of
-// mB.chi (chunk by chunk: the sum over chunks is linear), so the vec pass
-// multiplies each element of E and mA once: mZc = mC.chi + E.w + mA.(F.chi).
-// In Z_2^128 the vec pass keeps the three products (w = mB.chi): measured on
-// GB300, 160 us against 188 us for the 32768 x 576 x 64 layer's call, where the
-// Z_2^64 layers gain 2-5 % from the fold.
+// The two terms in E are one product: E.(mB.chi) + alpha * E.(F.chi) =
+// E.w with w = mB.chi + alpha * F.chi mod 2^(64 W) (the ring is commutative and
+// the sums distribute), so the vec pass multiplies each element of E and mA
+// once: mZc = mC.chi + E.w + mA.(F.chi).  The rows pass stores w in place of
+// mB.chi (chunk by chunk: the sum over chunks is linear), in Z_2^128 only for
+// layers with many rows: its 128-bit product, by one lane per row of K, costs
+// the rows pass 8 % on ResNet-18 at batch 1, and saves the vec pass 63 of 440 us
+// at batch 16.  Elsewhere the vec pass forms w as it goes.
 //
 // Up to three launches on the caller's stream:
 //   1. rows_kernel   one pass over the five N-wide matrices.  A warp owns a
@@ -20,11 +20,16 @@
 //                    mZ on the fly) or mB, F, and leaves per-chunk partial
 //                    dot products with chi in the workspace.  Each input word
 //                    is read from HBM exactly once.
-//   2. finalize_kernel  sums the K-side partials into the vectors w (or mB.chi), F.chi
+//   2. finalize_kernel  sums the K-side partials into the vectors w and F.chi
 //                    (only when a row is split into several chunks; with one
 //                    chunk the partials are those vectors and vec reads them).
-//   3. vec_kernel    one warp per output row: the two M x K GEMVs over E and
-//                    mA against those vectors, then mZc, mDc and Dc.
+//   3. vec_kernel    the two M x K GEMVs over E and mA against those vectors,
+//                    then mZc, mDc and Dc.  Several warps share a row (few
+//                    rows), or a warp takes four rows at a time, or eight lanes
+//                    a row (K < 64).
+// All passes are bound by memory; several rows per warp are what keeps enough
+// loads in flight where a row is short, and they share the loads of the vectors
+// and one reduction across lanes.
 // Every sum is a wrapping sum mod 2^(64 W), so the split into chunks does not
 // change any result bit.
 #include <new>
@@ -56,6 +61,31 @@ __device__ __forceinline__ typename Elem<W>::T warp_sum(typename Elem<W>::T v) {
         }
         return v;
     }
+}
+
+template <int W>
+__device__ __forceinline__ typename Elem<W>::T shfl_xor(typename Elem<W>::T v, int o) {
+    if constexpr (W == 1) {
+        return __shfl_xor_sync(0xffffffffu, v, o);
+    } else {
+        const u64 lo = __shfl_xor_sync(0xffffffffu, (u64)v, o), hi = __shfl_xor_sync(0xffffffffu, (u64)(v >> 64), o);
+        return (u128)lo | ((u128)hi << 64);
+    }
+}
+
+// Sums over the warp of four values per lane: the result for value
+// (lane >> 3) ends in every lane (halves are exchanged instead of summing each
+// value over all lanes: 6 shuffles of an element instead of 20).
+template <int W>
+__device__ __forceinline__ typename Elem<W>::T warp_sum4(const typename Elem<W>::T (&v)[4], int lane) {
+    using T = typename Elem<W>::T;
+    const bool h = lane & 16, q = lane & 8;
+    const T a = (h ? v[2] : v[0]) + shfl_xor<W>(h ? v[0] : v[2], 16);
+    const T b = (h ? v[3] : v[1]) + shfl_xor<W>(h ? v[1] : v[3], 16);
+    T r = (q ? b : a) + shfl_xor<W>(q ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) r += shfl_xor<W>(r, o);
+    return r;
 }
 
 struct Split {
@@ -107,12 +137,12 @@ struct RowsParams {
     const u64 *alpha, *mR, *Dt, *mC, *mB, *F, *chi;
     u64* mZ;   // NULL: the OptMAC tag is not written
     u64 *pmr, *pd, *pmc, *qmb, *qf;
-    int with_eu;   // the E.(F.chi) term is present (Z_2^64: folded into the K-side partial of mB.chi)
+    int fold;      // store w in place of mB.chi
 };
 
 // VEC = 2: two Z_2^64 elements per 16-byte access (needs even N).  Warp
 // task g of one layer.
-template <int W, int VEC>
+template <int W, int VEC, bool FOLD>
 __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int lane) {
     using T = typename Elem<W>::T;
     const int64_t tasksA = p.M * p.S, tasksB = p.K * p.S;
@@ -182,8 +212,8 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
         }
         s1 = warp_sum<W>(s1);
         s2 = warp_sum<W>(s2);
-        if (W == 1 && p.with_eu) s1 += alpha * s2;   // the chunk's part of w = mB.chi + alpha * F.chi
         if (lane == 0) {
+            if constexpr (FOLD) s1 += alpha * s2;   // the chunk's part of w = mB.chi + alpha * F.chi
             st_elem<W>(p.qmb, t, s1);
             st_elem<W>(p.qf, t, s2);
         }
@@ -194,7 +224,9 @@ template <int W, int VEC>
 __global__ void __launch_bounds__(NT) rows_kernel(RowsParams p) {
     ptx::grid_dep_launch();   // finalize and vec wait for this grid before reading
     ptx::grid_dep_wait();     // launched as a dependent of the kernel before it
-    rows_body<W, VEC>(p, (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5), threadIdx.x & 31);
+    const int64_t g = (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5);
+    if (p.fold) rows_body<W, VEC, true>(p, g, threadIdx.x & 31);
+    else rows_body<W, VEC, false>(p, g, threadIdx.x & 31);
 }
 
 template <int W>
@@ -223,23 +255,44 @@ __global__ void finalize_kernel(int64_t K, int64_t S, const u64* qmb, const u64*
 
 struct VecParams {
     int64_t M, K, S;
-    int with_eu;
-    const u64 *alpha, *E, *mA, *vmb, *vf, *pmr, *pd, *pmc;   // vmb: w (Z_2^64) or mB.chi (Z_2^128)
+    int form_w;    // vmb is mB.chi, and w is formed from it (FORM below)
+    const u64 *alpha, *E, *mA, *vmb, *vf, *pmr, *pd, *pmc;   // vmb: w, or mB.chi
     u64 *mDc, *Dc;
 };
 
-// `wpr` warps share one row (1, 2, 4 or 8), each taking every wpr-th chunk of
-// 32 (or 64, vectorised) K values; their partial sums meet in shared memory.
-template <int W, int VEC>
+// w_k from the stored vectors
+template <int W, bool FORM>
+__device__ __forceinline__ typename Elem<W>::T vec_w(typename Elem<W>::T b, typename Elem<W>::T u,
+                                                     typename Elem<W>::T alpha) {
+    if constexpr (FORM) return b + alpha * u;
+    else return b;
+}
+
+// acc = E.w + mA.(F.chi) of row r: the row's compact tag outputs
+template <int W>
+__device__ __forceinline__ void vec_store(const VecParams& p, int64_t r, typename Elem<W>::T acc) {
+    using T = typename Elem<W>::T;
+    T mrc = 0, dc = 0, mcc = 0;
+    for (int64_t s = 0; s < p.S; ++s) {
+        mrc += ld_elem<W>(p.pmr, r * p.S + s);
+        dc += ld_elem<W>(p.pd, r * p.S + s);
+        mcc += ld_elem<W>(p.pmc, r * p.S + s);
+    }
+    st_elem<W>(p.mDc, r, mrc - (mcc + acc));
+    st_elem<W>(p.Dc, r, dc);
+}
+
+// Few rows: `wpr` warps share one row (1, 2, 4 or 8), each taking every wpr-th
+// chunk of 32 (or 64, vectorised) K values; their sums meet in shared memory.
+template <int W, int VEC, bool FORM>
 __device__ __forceinline__ void vec_body(const VecParams& p, int wpr, int64_t blk) {
     using T = typename Elem<W>::T;
-    constexpr int NP = W == 1 ? 2 : 3;   // partial sums per row
-    __shared__ T part[NP][WARPS];
+    __shared__ T part[WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rows_per_block = WARPS / wpr;
     const int64_t r = blk * rows_per_block + warp / wpr;
     const int sub = warp % wpr;
-    T e_w = 0, ma_u = 0, e_u = 0;   // E.w, mA.(F.chi) and (Z_2^128) E.(F.chi) of row r
+    T acc = 0, am = 0;
     if (r < p.M) {
         const int64_t base = r * p.K;
         if constexpr (VEC == 2) {
@@ -249,100 +302,154 @@ __device__ __forceinline__ void vec_body(const VecParams& p, int wpr, int64_t bl
                 ulonglong2 ma = __ldg(reinterpret_cast<const ulonglong2*>(p.mA + base + k));
                 ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p.vmb + k);
                 ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p.vf + k);
-                e_w += e.x * w.x + e.y * w.y;
-                ma_u += ma.x * u.x + ma.y * u.y;
+                acc += e.x * w.x + e.y * w.y;
+                am += ma.x * u.x + ma.y * u.y;
             }
         } else {
-#pragma unroll 4
-            for (int64_t k = sub * 32 + lane; k < p.K; k += 32 * wpr) {
-                T e = ldg_elem<W>(p.E, base + k);
-                T ma = ldg_elem<W>(p.mA, base + k);
-                T w = ld_elem<W>(p.vmb, k);
-                T u = ld_elem<W>(p.vf, k);
-                e_w += e * w;
-                ma_u += ma * u;
-                if constexpr (W == 2) e_u += e * u;
+            // four chunks' loads together, zeros past the end
+            const int64_t step = 32 * wpr;
+            T eu = 0;
+            for (int64_t k = sub * 32 + lane; k < p.K; k += 4 * step) {
+                T e[4], a[4], w[4], u[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t j = k + i * step;
+                    const bool in = j < p.K;
+                    e[i] = in ? ldg_elem<W>(p.E, base + j) : (T)0;
+                    a[i] = in ? ldg_elem<W>(p.mA, base + j) : (T)0;
+                    w[i] = in ? ld_elem<W>(p.vmb, j) : (T)0;
+                    u[i] = in ? ld_elem<W>(p.vf, j) : (T)0;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc += e[i] * w[i];
+                    am += a[i] * u[i];
+                    if constexpr (FORM) eu += e[i] * u[i];
+                }
             }
+            // FORM: E.w = E.(mB.chi) + alpha * E.(F.chi), three independent sums
+            if constexpr (FORM) am += ld_elem<W>(p.alpha, 0) * eu;
         }
-        e_w = warp_sum<W>(e_w);
-        ma_u = warp_sum<W>(ma_u);
-        if constexpr (W == 2) e_u = warp_sum<W>(e_u);
+        acc = warp_sum<W>(acc + am);
     }
-    if (lane == 0) {
-        part[0][warp] = e_w;
-        part[1][warp] = ma_u;
-        if constexpr (W == 2) part[2][warp] = e_u;
-    }
+    if (lane == 0) part[warp] = acc;
     __syncthreads();
     if (r < p.M && sub == 0 && lane == 0) {
-        for (int j = 1; j < wpr; ++j) {
-            e_w += part[0][warp + j];
-            ma_u += part[1][warp + j];
-            if constexpr (W == 2) e_u += part[2][warp + j];
-        }
-        T mrc = 0, dc = 0, mcc = 0;
-        for (int64_t s = 0; s < p.S; ++s) {
-            mrc += ld_elem<W>(p.pmr, r * p.S + s);
-            dc += ld_elem<W>(p.pd, r * p.S + s);
-            mcc += ld_elem<W>(p.pmc, r * p.S + s);
-        }
-        T mzc = mcc + e_w + ma_u;
-        if (W == 2 && p.with_eu) mzc += ld_elem<W>(p.alpha, 0) * e_u;
-        st_elem<W>(p.mDc, r, mrc - mzc);
-        st_elem<W>(p.Dc, r, dc);
+        for (int j = 1; j < wpr; ++j) acc += part[warp + j];
+        vec_store<W>(p, r, acc);
     }
 }
 
+// Many rows: a warp takes four rows at a time, so that each load of the vectors
+// serves four rows and eight or more row loads are in flight per lane.
 template <int W, int VEC>
-__global__ void __launch_bounds__(NT) vec_kernel(VecParams p, int wpr) {
-    ptx::grid_dep_wait();   // the rows partials and the finalized vectors
-    vec_body<W, VEC>(p, wpr, blockIdx.x);
+__device__ __forceinline__ void vec4_body(const VecParams& p, int64_t blk) {
+    using T = typename Elem<W>::T;
+    const int lane = threadIdx.x & 31;
+    const int64_t r0 = (blk * WARPS + (threadIdx.x >> 5)) * 4;
+    if (r0 >= p.M) return;
+    T acc[4] = {0, 0, 0, 0};
+    int64_t base[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) base[i] = (r0 + i < p.M ? r0 + i : r0) * p.K;
+#pragma unroll(W == 1 ? 2 : 1)
+    for (int64_t k = VEC * lane; k < p.K; k += 32 * VEC) {
+        if constexpr (VEC == 2) {
+            ulonglong2 e[4], a[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                e[i] = ld_stream2(p.E + base[i] + k);
+                a[i] = ld_stream2(p.mA + base[i] + k);
+            }
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p.vmb + k);
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p.vf + k);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += e[i].x * w.x + e[i].y * w.y + a[i].x * u.x + a[i].y * u.y;
+        } else {
+            T e[4], a[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                e[i] = ldg_elem<W>(p.E, base[i] + k);
+                a[i] = ldg_elem<W>(p.mA, base[i] + k);
+            }
+            const T w = ld_elem<W>(p.vmb, k), u = ld_elem<W>(p.vf, k);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] += e[i] * w + a[i] * u;
+        }
+    }
+    const T v = warp_sum4<W>(acc, lane);
+    const int64_t r = r0 + (lane >> 3);
+    if ((lane & 7) == 0 && r < p.M) vec_store<W>(p, r, v);
 }
 
-// K < 64: one thread per row, the two compressed K-vectors staged in shared
-// memory (a warp per row would leave most lanes idle)
+// K < 64: eight lanes per row, four rows per lane group; a block covers 128 rows
 constexpr int SMALL_K = 64;
+constexpr int SMALL_ROWS = WARPS * 16;
 
-template <int W>
+template <int W, bool FORM>
 __device__ __forceinline__ void vec_small_body(const VecParams& p, int64_t blk) {
     using T = typename Elem<W>::T;
-    __shared__ T smb[SMALL_K], sf[SMALL_K];
-    for (int k = threadIdx.x; k < p.K; k += NT) {
-        smb[k] = ld_elem<W>(p.vmb, k);
-        sf[k] = ld_elem<W>(p.vf, k);
+    const int lane = threadIdx.x & 31, l = lane & 7, grp = lane >> 3;
+    const int64_t r0 = blk * SMALL_ROWS + (threadIdx.x >> 5) * 16;
+    const T alpha = FORM ? ld_elem<W>(p.alpha, 0) : (T)0;
+    T acc[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t r = r0 + i * 4 + grp;
+        if (r >= p.M) continue;
+#pragma unroll 4
+        for (int64_t k = l; k < p.K; k += 8) {
+            const T u = ld_elem<W>(p.vf, k);
+            acc[i] += ldg_elem<W>(p.E, r * p.K + k) * vec_w<W, FORM>(ld_elem<W>(p.vmb, k), u, alpha) +
+                      ldg_elem<W>(p.mA, r * p.K + k) * u;
+        }
     }
-    __syncthreads();
-    const int64_t r = blk * NT + threadIdx.x;
-    if (r >= p.M) return;
-    T e_w = 0, ma_u = 0, e_u = 0;
-    const int64_t base = r * p.K;
-    for (int k = 0; k < (int)p.K; ++k) {
-        const T e = ldg_elem<W>(p.E, base + k);
-        const T ma = ldg_elem<W>(p.mA, base + k);
-        e_w += e * smb[k];
-        ma_u += ma * sf[k];
-        if constexpr (W == 2) e_u += e * sf[k];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) acc[i] += shfl_xor<W>(acc[i], o);
+        const int64_t r = r0 + i * 4 + grp;
+        if (l == i && r < p.M) vec_store<W>(p, r, acc[i]);
     }
-    T mrc = 0, dc = 0, mcc = 0;
-    for (int64_t s = 0; s < p.S; ++s) {
-        mrc += ld_elem<W>(p.pmr, r * p.S + s);
-        dc += ld_elem<W>(p.pd, r * p.S + s);
-        mcc += ld_elem<W>(p.pmc, r * p.S + s);
-    }
-    T mzc = mcc + e_w + ma_u;
-    if (W == 2 && p.with_eu) mzc += ld_elem<W>(p.alpha, 0) * e_u;
-    st_elem<W>(p.mDc, r, mrc - mzc);
-    st_elem<W>(p.Dc, r, dc);
 }
 
-template <int W>
-__global__ void __launch_bounds__(NT) vec_small_kernel(VecParams p) {
-    ptx::grid_dep_wait();
-    vec_small_body<W>(p, blockIdx.x);
+// How the vec pass covers a layer's rows: eight lanes per row (K < 64), four
+// rows per warp with enough rows, else several warps per row.  Enough is four
+// such warps per SM in Z_2^64 (8192 x 1152: 34.6 -> 32.4 us) and in grouped
+// calls, whose other layers fill the SMs (ResNet-18 b16 in Z_2^128: 561 -> 377 us;
+// 445 us with the next bound), and 16 for a layer by itself in Z_2^128
+// (16384 x 576: 70 -> 64 us, but 4096 x 1152: 41 -> 57 us); four times as many
+// below K = 512, where a row is short (5880 x 207: 3 us slower).
+enum VecMode { VEC_SMALL, VEC_FOUR, VEC_SHARED };
+VecMode vec_mode(int64_t M, int64_t K, bool alone128) {
+    return K < SMALL_K ? VEC_SMALL : M >= 4 * 152 * (alone128 || K < 512 ? 16 : 4) ? VEC_FOUR : VEC_SHARED;
+}
+
+// the rows pass stores w for this layer
+template <int W> bool folds(VecMode mode) { return W == 1 || mode == VEC_FOUR; }
+
+template <int W, int VEC, int MODE, bool FORM>
+__global__ void __launch_bounds__(NT) vec_kernel(VecParams p, int wpr) {
+    ptx::grid_dep_wait();   // the rows partials and the finalized vectors
+    if constexpr (MODE == VEC_SMALL) vec_small_body<W, FORM>(p, blockIdx.x);
+    else if constexpr (MODE == VEC_FOUR) vec4_body<W, VEC>(p, blockIdx.x);
+    else vec_body<W, VEC, FORM>(p, wpr, blockIdx.x);
 }
 
 int vec_warps_per_row(int64_t K) {
     return K >= 2048 ? 8 : K >= 1024 ? 4 : K >= 256 ? 2 : 1;
+}
+
+// blocks of the vec pass
+int64_t vec_blocks(int64_t M, int64_t K, bool alone128) {
+    switch (vec_mode(M, K, alone128)) {
+        case VEC_SMALL: return (M + SMALL_ROWS - 1) / SMALL_ROWS;
+        case VEC_FOUR: return (M + 4 * WARPS - 1) / (4 * WARPS);
+        default: {
+            const int64_t rpb = WARPS / vec_warps_per_row(K);
+            return (M + rpb - 1) / rpb;
+        }
+    }
 }
 
 template <int W>
@@ -351,7 +458,9 @@ cudaError_t run(const CompactArgs& a, char* ws, cudaStream_t st) {
     WsLayout L = ws_layout(a.M, a.K, a.N, W);
     RowsParams rp{a.M, a.K, a.N, sp.S, sp.cw, a.alpha, a.mR, a.Dt, a.mC, a.mB, a.F, a.chi, a.mZ,
                   (u64*)(ws + L.pmr), (u64*)(ws + L.pd), (u64*)(ws + L.pmc),
-                  (u64*)(ws + L.qmb), (u64*)(ws + L.qf), a.with_eu};
+                  (u64*)(ws + L.qmb), (u64*)(ws + L.qf), 0};
+    const VecMode mode = vec_mode(a.M, a.K, W == 2);
+    rp.fold = a.with_eu && folds<W>(mode);
     const int64_t tasks = (a.M + a.K) * sp.S;
     if (tasks > 0) {
         const unsigned blocks = (unsigned)((tasks + WARPS - 1) / WARPS);
@@ -371,21 +480,20 @@ cudaError_t run(const CompactArgs& a, char* ws, cudaStream_t st) {
                                                (u64*)(ws + L.vf));
         if (e != cudaSuccess) return e;
     }
-    VecParams vp{a.M, a.K, sp.S, a.with_eu, a.alpha, a.E, a.mA, fin ? (const u64*)(ws + L.vmb) : rp.qmb,
+    VecParams vp{a.M, a.K, sp.S, a.with_eu && !rp.fold, a.alpha, a.E, a.mA, fin ? (const u64*)(ws + L.vmb) : rp.qmb,
                  fin ? (const u64*)(ws + L.vf) : rp.qf, rp.pmr, rp.pd, rp.pmc, a.mDc, a.Dc};
-    if (a.K < SMALL_K) {
-        const cudaError_t e =
-            launch_dependent(vec_small_kernel<W>, dim3((unsigned)((a.M + NT - 1) / NT)), dim3(NT), 0, st, vp);
-        if (e != cudaSuccess) return e;
-    } else {
-        const int wpr = vec_warps_per_row(a.K);
-        const int64_t rpb = WARPS / wpr;
-        const unsigned vb = (unsigned)((a.M + rpb - 1) / rpb);
-        const cudaError_t e = W == 1 && (a.K % 2) == 0
-                                  ? launch_dependent(vec_kernel<W, 2>, dim3(vb), dim3(NT), 0, st, vp, wpr)
-                                  : launch_dependent(vec_kernel<W, 1>, dim3(vb), dim3(NT), 0, st, vp, wpr);
-        if (e != cudaSuccess) return e;
-    }
+    const bool vec2 = W == 1 && (a.K % 2) == 0;
+    constexpr int V = 3 - W;      // elements per access where K is even
+    constexpr bool F = W == 2;    // Z_2^128 may form w
+    auto* kernel =
+        mode == VEC_SMALL  ? (vp.form_w ? vec_kernel<W, 1, VEC_SMALL, F> : vec_kernel<W, 1, VEC_SMALL, false>)
+        : mode == VEC_FOUR ? (vec2 ? vec_kernel<W, V, VEC_FOUR, false> : vec_kernel<W, 1, VEC_FOUR, false>)
+        : vp.form_w        ? vec_kernel<W, 1, VEC_SHARED, F>
+        : vec2             ? vec_kernel<W, V, VEC_SHARED, false>
+                           : vec_kernel<W, 1, VEC_SHARED, false>;
+    const cudaError_t e = launch_dependent(kernel, dim3((unsigned)vec_blocks(a.M, a.K, W == 2)), dim3(NT), 0, st, vp,
+                                           vec_warps_per_row(a.K));
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -400,7 +508,7 @@ struct CompactLayer {
     RowsParams rp;
     VecParams vp;
     int rows_vec2;   // rows pass on 16-byte pairs
-    int vec_small;   // K < SMALL_K: one thread per row
+    int vec_mode;
     int vec_vec2;    // vec pass on 16-byte pairs
     int wpr;         // warps per row in the vec pass
     u64 *vmb, *vf;
@@ -432,8 +540,14 @@ __global__ void __launch_bounds__(NT) rows_group_kernel(const __grid_constant__ 
     const int li = layer_of(g.rb, g.count, blockIdx.x);
     const CompactLayer& L = g.L[li];
     const int64_t task = ((int64_t)blockIdx.x - g.rb[li]) * WARPS + (threadIdx.x >> 5);
-    if (W == 1 && L.rows_vec2) rows_body<W, 2>(L.rp, task, threadIdx.x & 31);
-    else rows_body<W, 1>(L.rp, task, threadIdx.x & 31);
+    const int lane = threadIdx.x & 31;
+    if (L.rp.fold) {
+        if (W == 1 && L.rows_vec2) rows_body<W, 2, true>(L.rp, task, lane);
+        else rows_body<W, 1, true>(L.rp, task, lane);
+    } else {
+        if (W == 1 && L.rows_vec2) rows_body<W, 2, false>(L.rp, task, lane);
+        else rows_body<W, 1, false>(L.rp, task, lane);
+    }
 }
 
 template <int W>
@@ -448,17 +562,20 @@ __global__ void __launch_bounds__(256) finalize_group_kernel(const __grid_consta
 }
 
 template <int W>
-__global__ void __launch_bounds__(NT) vec_group_kernel(const __grid_constant__ CompactGroup g) {
+__global__ void __launch_bounds__(NT, 3) vec_group_kernel(const __grid_constant__ CompactGroup g) {
     ptx::grid_dep_wait();
     const int li = layer_of(g.vb, g.count, blockIdx.x);
     const CompactLayer& L = g.L[li];
     const int64_t blk = (int64_t)blockIdx.x - g.vb[li];
-    if (L.vec_small) vec_small_body<W>(L.vp, blk);
-    else if (W == 1 && L.vec_vec2) vec_body<W, 2>(L.vp, L.wpr, blk);
-    else vec_body<W, 1>(L.vp, L.wpr, blk);
+    const bool vec2 = W == 1 && L.vec_vec2;
+    constexpr bool F = W == 2;
+    if (L.vec_mode == VEC_SMALL) L.vp.form_w ? vec_small_body<W, F>(L.vp, blk) : vec_small_body<W, false>(L.vp, blk);
+    else if (L.vec_mode == VEC_FOUR) vec2 ? vec4_body<W, 3 - W>(L.vp, blk) : vec4_body<W, 1>(L.vp, blk);
+    else if (L.vp.form_w) vec_body<W, 1, F>(L.vp, L.wpr, blk);
+    else vec2 ? vec_body<W, 3 - W, false>(L.vp, L.wpr, blk) : vec_body<W, 1, false>(L.vp, L.wpr, blk);
 }
 
-// blocks of each kernel for one layer
+// blocks of each kernel for one layer of a group
 struct CompactBlocks {
     int64_t rows, fin, vec;
 };
@@ -472,12 +589,7 @@ CompactBlocks compact_blocks(int64_t M, int64_t K, int64_t N) {
         b.fin = (K + 255) / 256;
         if (b.fin > 1024) b.fin = 1024;
     }
-    if (K < SMALL_K) {
-        b.vec = (M + NT - 1) / NT;
-    } else {
-        const int64_t rpb = WARPS / vec_warps_per_row(K);
-        b.vec = (M + rpb - 1) / rpb;
-    }
+    b.vec = vec_blocks(M, K, false);
     return b;
 }
 
@@ -499,16 +611,18 @@ cudaError_t run_group(const CompactArgs* a, int n, char* const* ws, cudaStream_t
             CompactLayer& L = g->L[cnt];
             L.rp = RowsParams{x.M, x.K, x.N, sp.S, sp.cw, x.alpha, x.mR, x.Dt, x.mC, x.mB, x.F, x.chi, x.mZ,
                               (u64*)(w + wl.pmr), (u64*)(w + wl.pd), (u64*)(w + wl.pmc),
-                              (u64*)(w + wl.qmb), (u64*)(w + wl.qf), x.with_eu};
+                              (u64*)(w + wl.qmb), (u64*)(w + wl.qf), 0};
+            const VecMode mode = vec_mode(x.M, x.K, false);
+            L.rp.fold = x.with_eu && folds<W>(mode);
             L.vmb = (u64*)(w + wl.vmb);
             L.vf = (u64*)(w + wl.vf);
             // one chunk per row: the vec pass reads the partials in place (no finalize blocks)
             const bool fin = x.K > 0 && sp.S > 1;
-            L.vp = VecParams{x.M, x.K, sp.S, x.with_eu, x.alpha, x.E, x.mA, fin ? L.vmb : L.rp.qmb,
+            L.vp = VecParams{x.M, x.K, sp.S, x.with_eu && !L.rp.fold, x.alpha, x.E, x.mA, fin ? L.vmb : L.rp.qmb,
                              fin ? L.vf : L.rp.qf, L.rp.pmr, L.rp.pd,
                              L.rp.pmc, x.mDc, x.Dc};
             L.rows_vec2 = (x.N % 2) == 0;
-            L.vec_small = x.K < SMALL_K;
+            L.vec_mode = mode;
             L.vec_vec2 = (x.K % 2) == 0;
             L.wpr = vec_warps_per_row(x.K);
             const CompactBlocks b = compact_blocks(x.M, x.K, x.N);
