@@ -438,13 +438,12 @@ size_t region(const mpc_layer& L, bool with_crt) {
     return (b + 255) & ~size_t(255);
 }
 
-// In a group, Z_2^64 layers that the digit tiles can run stay with them unless
-// the table says otherwise: they share one launch pair with the group's other
-// layers, where a layer on the residue path runs by itself (48 uneven layers:
-// 1427 us per step with the digits, 1421 us with the rule's three layers on the
-// residue path).
+// The residue path in a group: a layer there runs by itself, where the digit
+// tiles share their launches, so the rule asks for a larger gain.  Z_2^64 layers
+// that the digit tiles can run stay with them unless the table says otherwise.
 bool group_uses_crt(const mpcl::Choice& c, int64_t M, int64_t K, int64_t N, int words) {
-    return c.crt && (c.tuned || words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words));
+    if (!c.crt || c.tuned) return c.crt != 0;
+    return (words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words)) && mpcl::gemm_crt_preferred(M, K, N, words, true);
 }
 
 size_t group_gemm_ws(const mpc_layer* layers, int count, bool with_crt) {

@@ -960,9 +960,12 @@ CrtPlan crt_plan(int64_t M, int64_t K, int64_t N, int words, int one_half) {
             q.kps = kps;
         }
     }
-    // the GEMM reads every plane from memory once; splitting the operands
-    q.us = std::max(q.us, (double)(q.a_mod + q.b_mod) * q.np * 1.6e-7) +
-           (double)(q.a_tiles * 128 + q.b_tiles * (q.bn / 2)) * q.kb * KB * (words == 1 ? 7.6e-6 : 17.4e-6) + 14.0;
+    // estimate of the whole call, fitted to 45 share calls per ring (mean error 6-7 %)
+    const double el = (double)(q.a_tiles * 128 + q.b_tiles * (q.bn / 2)) * q.kb * KB;
+    const double stages = (double)cdiv(T * q.splits, 76) * q.kps * q.bn / 256;
+    const double res = (double)q.splits * q.mt * q.nt * TM * q.bn * q.np;
+    q.us = words == 1 ? 14.4 + 1.01e-5 * el + 0.293 * stages + 1.15e-6 * res
+                      : 12.9 + 2.25e-5 * el + 0.209 * stages + 0.80e-6 * res;
     auto up = [](int64_t b) { return (size_t)((b + 255) / 256 * 256); };
     q.off_b = up(q.a_mod * q.np);
     q.off_res = q.off_b + up(q.b_mod * q.np);
@@ -1047,23 +1050,30 @@ bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half)
            (double)q.mt * q.nt * (q.bn / 8) * 2 < 2e9;
 }
 
-// Estimated time of the other paths: the digit tiles at their measured rates
-// (2 M K N ring multiply-adds: 19.5 per ps in Z_2^64, 4.3 in Z_2^128, on 128-row
-// and 32- or 16-column tiles), or the integer pipes (2.1) for the Z_2^64 layers
-// with odd N that the digit tiles do not take.
+// Estimated time of the other paths, fitted to the same calls: the digit tiles
+// (a constant, the left operand's digit planes, and the waves of Kd-deep units
+// over 152 SMs), or the integer pipes for the Z_2^64 layers with odd N that the
+// digit tiles do not take.
 namespace {
 double digit_us(int64_t M, int64_t K, int64_t N, int words) {
-    if (!gemm_tc_feasible(M, K, N, words)) return 5.0 + 2.0 * M * K * N / (words == 1 ? 2.1e6 : 0.5e6);
-    const int nd = words == 1 ? 32 : 16, rows = M <= 64 ? 64 : 128;
-    return 12.0 + 2.0 * cdiv(M, rows) * rows * K * cdiv(N, nd) * nd / (words == 1 ? 19.5e6 : 4.3e6);
+    if (!gemm_tc_feasible(M, K, N, words)) return 15.0 + 2.0 * M * K * N / (words == 1 ? 2.15e6 : 0.5e6);
+    const int64_t nd = words == 1 ? 32 : 16, kd = words == 1 ? 128 : 64;
+    const int64_t U = cdiv(M, 128) * cdiv(N, nd) * cdiv(2 * cdiv(K, KS) * KS, kd);
+    const double mb = 2.0 * M * K * 16e-6 * words;
+    return words == 1 ? 14.9 + 0.127 * mb + 0.43 * cdiv(U, 152) + 3.51 * U / 152
+                      : 21.5 + 0.216 * mb + 1.91 * cdiv(U, 152) + 1.86 * U / 152;
 }
 constexpr size_t MAX_WORKSPACE = size_t(12) << 30;
-// The residue path's time over the other paths'
-double crt_ratio(int64_t M, int64_t K, int64_t N, int words) {
+// The residue path's time over the other paths'.  In a group the digit tiles'
+// launch, set-up and last wave are shared with the other layers.
+double crt_ratio(int64_t M, int64_t K, int64_t N, int words, bool grouped = false) {
     if (M <= 8 || N <= 8 || !gemm_crt_feasible(M, K, N, words, 0)) return 1e9;
+    // up to 64 rows the wide and 64-row digit tiles waste less than 256-row tiles
+    if (M <= 64 && gemm_tc_feasible(M, K, N, words)) return 1e8;
     const CrtPlan q = crt_plan(M, K, N, words, 0);
     if (q.total > MAX_WORKSPACE) return 1e9;
-    return q.us / digit_us(M, K, N, words);
+    const double shared = grouped ? (words == 1 ? 12.0 : 18.0) : 0.0;
+    return q.us / (digit_us(M, K, N, words) - shared);
 }
 }  // namespace
 
@@ -1073,7 +1083,9 @@ bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words) {
     const double r = crt_ratio(M, K, N, words);
     return r < 1.1 || (r < 1e9 && crt_plan(M, K, N, words, 0).total <= (size_t(32) << 20));
 }
-bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words) { return crt_ratio(M, K, N, words) < 0.95; }
+bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words, bool grouped) {
+    return M > 32 && N > 64 && crt_ratio(M, K, N, words, grouped) < 0.93;   // within the measured sizes
+}
 
 size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_half) {
     return crt_plan(M, K, N, words, one_half).total;

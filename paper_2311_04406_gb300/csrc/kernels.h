@@ -81,7 +81,7 @@ int tc_timeout_flag(bool* set);   // synchronous; 0 on success
 // superset of the shapes the built-in rule runs on it.
 bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
 bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words);
-bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words);
+bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words, bool grouped = false);
 size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
 constexpr int CRT_LAUNCHES = 3;
 cudaError_t launch_gemm_crt(const GemmArgs& a, void* ws, size_t ws_bytes, cudaStream_t st);
