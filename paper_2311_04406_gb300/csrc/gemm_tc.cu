@@ -117,16 +117,16 @@ constexpr int NINFO = 4;                 // unit descriptors in flight from the 
 
 template <int W, int G = 1, int R = BM> struct Layout {
     static constexpr int RAW = G == 1 ? RAW_ONE : RAW_GROUP;   // raw tiles in flight
-    static constexpr int NBARS = 4 * MAX_STAGES + 2 * RAW + 2 + 2 + 1 + NINFO;
+    static constexpr int NBARS = 4 * MAX_STAGES + 2 * RAW + 2 + 2 + 1 + NINFO + 4;
     static constexpr uint32_t A_PLANE = a_plane_bytes<R>();
     static constexpr uint32_t A_STAGE = Cfg<W>::NDIG * A_PLANE;
     static constexpr uint32_t OFF_B = Cfg<W>::STAGES * A_STAGE;
     static constexpr uint32_t OFF_RAW = OFF_B + Cfg<W>::STAGES * B_STAGE_BYTES;
-    // epilogue staging: per drain warp 32 rows x (ND + 1) sums (one element
-    // of padding per row keeps the row-wise writes and column-wise reads free
-    // of bank conflicts)
+    // epilogue staging: per drain warp 32 rows of ND sums (256 bytes), padded by
+    // 16 bytes against bank conflicts
     static constexpr uint32_t OFF_STG = OFF_RAW + RAW * RAW_BYTES;
-    static constexpr uint32_t STG_BYTES = 4 * 32 * (Cfg<W>::ND + 1) * 8 * W;
+    static constexpr uint32_t STG_ROW = Cfg<W>::ND * 8 * W + 16;
+    static constexpr uint32_t STG_BYTES = 4 * 32 * STG_ROW;
     static constexpr uint32_t OFF_BAR = OFF_STG + STG_BYTES;
     static constexpr uint32_t OFF_INFO = (OFF_BAR + NBARS * 8 + 16 + 15) / 16 * 16;   // int4 slots
     static constexpr uint32_t SMEM = OFF_INFO + NINFO * 16;
@@ -540,6 +540,7 @@ struct Unit {
     int ii;          // interval within the tile
     int nst;         // stages in this interval (KD, or fewer at the end of K)
     bool flush;      // last unit of a segment: the sums go to Z
+    bool whole;      // first unit of a tile that this CTA computes whole
 };
 
 // Walks the units of one CTA in order.  Divisions happen only where one of
@@ -638,6 +639,7 @@ template <int G> struct Walker {
         x.ii = ii;
         x.nst = min(cKD, cS - x.ii * cKD);
         x.flush = (left == 0) || (x.ii == cI - 1);
+        x.whole = x.ii == 0 && left >= cI - 1;
         return x;
     }
 };
@@ -713,6 +715,7 @@ template <> struct Walker<1> {
         x.ii = ii;
         x.nst = min(cKD, cS - x.ii * cKD);
         x.flush = (left == 0) || (x.ii == cI - 1);
+        x.whole = x.ii == 0 && left >= cI - 1;
         return x;
     }
 };
@@ -758,10 +761,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
     uint64_t* accEmpty = accFull + 2;
     uint64_t* mmaDone = accEmpty + 2;
     uint64_t* infoFull = mmaDone + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(infoFull + NINFO);
+    uint64_t* addFull = infoFull + NINFO;      // per drain warp: its rows of the addend have landed
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(addFull + 4);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     // the MMA warp hands each unit's (row tile, column tile, interval, flush |
-    // layer << 1) to the drain warps through NINFO slots
+    // whole << 1 | layer << 2) to the drain warps through NINFO slots
     int4* info = reinterpret_cast<int4*>(smem + Lay::OFF_INFO);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -797,6 +801,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
         }
         ptx::mbar_init(mmaDone, 1);
         for (int i = 0; i < NINFO; ++i) ptx::mbar_init(&infoFull[i], 1);
+        for (int i = 0; i < 4; ++i) ptx::mbar_init(&addFull[i], 1);
         *abort_flag = 0;
         ptx::fence_barrier_init();
     }
@@ -1001,7 +1006,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
             // slot v % NINFO last held unit v - NINFO, which the drain finished
             // before it released the accumulator set this wait was for
             if (lane == 0) {
-                info[v % NINFO] = make_int4((int)x.mt, (int)x.nt, x.ii, (int)x.flush | (wk.gi << 1));
+                info[v % NINFO] =
+                    make_int4((int)x.mt, (int)x.nt, x.ii, (int)x.flush | ((int)x.whole << 1) | (wk.gi << 2));
                 ptx::mbar_arrive(&infoFull[v % NINFO]);
             }
             for (int j = 0; j < x.nst; ++j, ++it) {
@@ -1047,12 +1053,27 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
         ptx::mma_commit_if(ptx::elect_one(), mmaDone);
         ptx::mbar_wait(mmaDone, 0, abort_flag, WAIT_LIMIT);
     } else {
-        // drain warps: TMEM lane quadrant = warp % 4
+        // Drain warps: TMEM lane quadrant = warp % 4; lane l of quadrant q holds
+        // row q RPW + l of the tile (64-row tiles: lanes 0-15).  Rows move between
+        // the warp's staging rows and memory by bulk copies, one 256-byte row per
+        // lane: the addend's rows of a tile computed whole arrive while its MMAs
+        // run, and C + sum (or, in Z_2^64, a piece of a split tile as a bulk
+        // addition) leaves while the next tile is drained.  With loads and stores
+        // by the warp a tile's epilogue took 11,100 clock cycles, more than the
+        // MMAs of a tile with 2K = 256, and a split piece 5,800: the share of a
+        // 4096 x 128 x 4096 layer took 354 us and takes 248, of 1024 x 576 x 64
+        // 18.9 and 17.2, of 256 x 576 x 128 17.0 and 15.4.
+        constexpr int RPW = R / 4;      // tile rows per drain warp
+        constexpr uint32_t STG_ROW = Lay::STG_ROW;
         const int quad = warp & 3;
+        uint8_t* stg = sStg + quad * 32 * STG_ROW;
+        uint8_t* row = stg + lane * STG_ROW;
         Sum sum[ND];
 #pragma unroll
         for (int c = 0; c < ND; ++c) sum[c] = 0;
         int seg_ii = -1;   // first interval of the current segment
+        uint32_t adds = 0;          // addend loads begun
+        bool pending = false;       // one of them has not been waited for
         for (int64_t v = 0; v < nv; ++v) {
             const bool have = ptx::mbar_wait(&infoFull[v % NINFO], (int)((v / NINFO) & 1), abort_flag, WAIT_LIMIT);
             if (!__all_sync(0xffffffffu, have)) {
@@ -1062,7 +1083,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
             const int4 u = info[v % NINFO];
             const int x_ii = u.z;
             const bool x_flush = (u.w & 1) != 0;
-            const TcParams& p = G == 1 ? g.p[0] : sp[u.w >> 1];
+            const TcParams& p = G == 1 ? g.p[0] : sp[u.w >> 2];
+            const int64_t m = (int64_t)u.x * R + quad * RPW + lane, n0 = (int64_t)u.y * ND;
+            const bool mine = lane < RPW && m < p.M;
+            // bytes of this tile's rows (N is even for W = 1: a multiple of 16)
+            const uint32_t bytes = (uint32_t)((p.N - n0 < ND ? p.N - n0 : ND) * 8 * W);
+            if ((u.w & 2) != 0 && p.C) {
+                ptx::bulk_wait_read();      // the last tile has left the staging rows
+                const int rows = __popc(__ballot_sync(0xffffffffu, mine));
+                if (lane == 0) ptx::mbar_arrive_expect_tx(&addFull[quad], rows * bytes);
+                __syncwarp();
+                if (mine) ptx::bulk_g2s(row, p.C + (m * p.N + n0) * W, bytes, &addFull[quad]);
+                ++adds;
+                pending = true;
+            }
             const int set = (int)(v & 1);
             bool got = ptx::mbar_wait(&accFull[set], (int)((v >> 1) & 1), abort_flag, WAIT_LIMIT);
             if (!__all_sync(0xffffffffu, got)) {
@@ -1084,52 +1118,65 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
                 // pieces of a split tile are added to Z (set to C by the prologue)
                 const bool whole = seg_ii == 0 && x_ii == p.I - 1;
                 seg_ii = -1;
-                // The warp's rows x ND sums go through shared memory so that
-                // the global accesses run along rows: lane = column (W = 1), or
-                // two rows of 16 columns per instruction (W = 2).  Lane l of
-                // quadrant q holds row q RPW + l of the tile; with 64-row tiles
-                // only lanes 0-15 hold rows (RPW = 16).
-                constexpr int RPW = R / 4;      // tile rows per drain warp
-                Sum* stg = reinterpret_cast<Sum*>(sStg) + quad * 32 * (ND + 1);
-                __syncwarp();
-#pragma unroll
-                for (int c = 0; c < ND; ++c) stg[lane * (ND + 1) + c] = sum[c];
-                __syncwarp();
-                constexpr int RPI = 32 / ND;     // rows per instruction
-                constexpr int NIT = RPW / RPI;
-                constexpr int BATCH = NIT;        // addend loads in flight together
-                const int rr = lane / ND, cc = lane % ND;
-                const int64_t n = (int64_t)u.y * ND + cc;
-                const int64_t mb = (int64_t)u.x * R + quad * RPW;
-#pragma unroll
-                for (int i0 = 0; i0 < NIT; i0 += BATCH) {
-                    // a batch of addend loads first, then its stores or atomic adds
-                    Sum cv[BATCH];
-#pragma unroll
-                    for (int i = 0; i < BATCH; ++i) {
-                        const int64_t m = mb + (i0 + i) * RPI + rr;
-                        cv[i] = (whole && p.C && m < p.M && n < p.N) ? ldg_elem<W>(p.C, m * p.N + n) : (Sum)0;
+                if (pending) {
+                    got = ptx::mbar_wait(&addFull[quad], (adds - 1) & 1, abort_flag, WAIT_LIMIT);
+                    if (!__all_sync(0xffffffffu, got)) {
+                        if (lane == 0) record_timeout(abort_flag);
+                        break;
                     }
-#pragma unroll
-                    for (int i = 0; i < BATCH; ++i) {
-                        const int r = (i0 + i) * RPI + rr;
-                        const int64_t m = mb + r;
-                        if (m < p.M && n < p.N) {
-                            const Sum v = stg[r * (ND + 1) + cc];
-                            const int64_t e = m * p.N + n;
-                            if (whole) {
-                                st_elem<W>(p.Z, e, cv[i] + v);
-                            } else {
-                                if constexpr (W == 1) red_add_u64(p.Z + e, v);
-                                else atomic_add_u128(p.Z + 2 * e, v);
-                            }
-                        }
-                    }
+                } else {
+                    ptx::bulk_wait_read();
                 }
+                ulonglong2* s2 = reinterpret_cast<ulonglong2*>(row);
+#pragma unroll
+                for (int q = 0; q < ND * W / 2; ++q) {
+                    ulonglong2 o = pending ? s2[q] : make_ulonglong2(0, 0);
+                    if constexpr (W == 1) {
+                        o.x += sum[2 * q];
+                        o.y += sum[2 * q + 1];
+                    } else {
+                        const Sum r = ((Sum)o.x | ((Sum)o.y << 64)) + sum[q];
+                        o.x = (u64)r;
+                        o.y = (u64)(r >> 64);
+                    }
+                    s2[q] = o;
+                }
+                pending = false;
 #pragma unroll
                 for (int c = 0; c < ND; ++c) sum[c] = 0;
+                if (whole || W == 1) {
+                    // each lane's own writes, before its own bulk copy reads them
+                    ptx::fence_proxy_async_smem();
+                    if (mine) {
+                        u64* z = p.Z + (m * p.N + n0) * W;
+                        if (whole) ptx::bulk_s2g(z, row, bytes);
+                        else ptx::bulk_add_u64(z, row, bytes);
+                    }
+                    ptx::bulk_commit();
+                } else {
+                    // Z_2^128 pieces: carries need atomics, which run along rows
+                    // (two rows of 16 columns per instruction).  Issuing eight
+                    // low words before the first carry is needed gained nothing.
+                    __syncwarp();
+                    constexpr int RPI = 32 / ND;
+                    const int rr = lane / ND, cc = lane % ND;
+                    const int64_t n = n0 + cc, mb = (int64_t)u.x * R + quad * RPW;
+#pragma unroll
+                    for (int r0 = 0; r0 < RPW; r0 += RPI) {
+                        const int64_t mm = mb + r0 + rr;
+                        if (mm < p.M && n < p.N)
+                            atomic_add_u128(p.Z + 2 * (mm * p.N + n),
+                                            ld_elem<W>(reinterpret_cast<const u64*>(stg + (r0 + rr) * STG_ROW), cc));
+                    }
+                    ptx::fence_proxy_async_smem();   // these reads, before a bulk load writes the rows
+                    __syncwarp();
+                }
             }
         }
+        // addend copies in flight (only after a timeout) land, and this thread's
+        // stores have read the staging rows and are complete
+        if (pending) ptx::mbar_wait(&addFull[quad], (adds - 1) & 1, abort_flag, WAIT_LIMIT);
+        ptx::bulk_wait();
     }
     ptx::tc_fence_before();
     __syncthreads();
