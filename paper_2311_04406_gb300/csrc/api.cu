@@ -90,7 +90,7 @@ int run_gemm(mpcl::GemmArgs g, void* ws, size_t ws_bytes, cudaStream_t st) {
     }
     g.simt_waves = c.waves;
     g.rows = c.rows;
-    return cuda_status(mpcl::launch_gemm_simt(g, st));
+    return cuda_status(mpcl::launch_gemm_simt(g, st, true));
 }
 
 }  // namespace
@@ -546,7 +546,7 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
     if (!side) {
         if (!tc.empty()) CHK(cuda_status(mpcl::launch_gemm_tc_grouped(tc.data(), (int)tc.size(), ap.data(), st)));
         CHK(run_crt());
-        for (const auto& x : simt) CHK(cuda_status(mpcl::launch_gemm_simt(x, st)));
+        for (const auto& x : simt) CHK(cuda_status(mpcl::launch_gemm_simt(x, st, true)));
         return MPC_OK;
     }
     std::lock_guard<std::mutex> lk(side->mu);
@@ -558,7 +558,7 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
     // stream; the first error is reported
     int status = MPC_OK;
     for (size_t j = 0; j < simt.size() && status == MPC_OK; ++j)
-        status = cuda_status(mpcl::launch_gemm_simt(simt[j], side->s[j % ns]));
+        status = cuda_status(mpcl::launch_gemm_simt(simt[j], side->s[j % ns], false));
     if (status == MPC_OK && !tc.empty())
         status = cuda_status(mpcl::launch_gemm_tc_grouped(tc.data(), (int)tc.size(), ap.data(), st));
     if (status == MPC_OK) status = run_crt();

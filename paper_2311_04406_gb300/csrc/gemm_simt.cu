@@ -6,22 +6,35 @@
 // to amortise a 128-row MMA tile, and skinny layers (M <= 8, e.g. dense layers
 // at batch 1) whose cost is streaming [B ; F] from memory.
 //
-// Two kernels, both optionally split along K over grid.z:
-//   * ring_gemm_simt_kernel<W, TM>: TM x 64 outputs per 256-thread block
-//     (TM = 64, or 16 for layers whose 64-row tiles would leave most SMs
+// Three kernels, all optionally split along K over grid.z:
+//   * ring_gemm_simt_kernel<W, TM, CLUSTER, J>: TM x 64 outputs per 256-thread
+//     block (TM = 64, or 16 for layers whose 64-row tiles would leave most SMs
 //     idle), 16-deep K slices staged in shared memory, each thread owns a
-//     (TM / 16) x 4 strided sub-tile (conflict-free shared reads).
-//   * ring_gemv_kernel (M <= 8): one thread per output column keeps M sums;
-//     the M rows of the left operand are staged in shared memory per K chunk
-//     and the right operand is read once, coalesced along N.  For narrow
-//     layers (N <= 256) ring_gemv_narrow_kernel instead has a block's eight
-//     warps take interleaved rows of its K range and add their sums up in
-//     shared memory, so that a block contributes one partial per output.
-// With a K split, Z is first set to C (a device-to-device copy) and every
-// block adds its partial sums with exact wrapping atomics; without one, the
-// block writes C + sum.  Out-of-range rows/columns/K are zero-filled.
+//     (TM / 16) x J strided sub-tile (conflict-free shared reads); J = 1 for
+//     layers of at most 16 columns.
+//   * ring_gemv_kernel (M <= 8): a block's eight warps take interleaved rows of
+//     its K range for 32 or 64 output columns and add their sums up in shared
+//     memory, so that a block contributes one partial per output.
+//   * ring_gemv_wide_kernel (M <= 8, wide layers with a long K): one thread per
+//     output column or pair keeps M sums; the right operand is read once,
+//     coalesced along N.
+// The K splits of an output that fit one thread-block cluster (of up to 16) are
+// added up through distributed shared memory: one launch, nothing set up before
+// it.  With more of them, Z is first set to C (a device-to-device copy) and
+// every block adds its partial sums with exact wrapping atomics.  Without a
+// split the block writes C + sum.  Out-of-range rows/columns/K are zero-filled.
+//
+// A block's time goes with its K slices (a 16-deep one takes about 1 us in
+// Z_2^64, 3-4 us in Z_2^128: the low 64 or 128 bits of a product need 1 or 6
+// wide multiply-adds, which issue at 15 per clock cycle and SM), so small layers
+// spread K over as many blocks as fit the chip once.  Shares before and now, us:
+// 64 x 128 x 64 11.1, 4.5 (Z_2^128: 17.9, 8.4); 33 x 70 x 40 9.3, 4.4; 16 x 512 x 10
+// 11.2, 6.0; 8 x 299 x 368 12.4, 8.0 (18.5, 10.0); 16 x 50000 x 10 57.9, 25.9.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
+#include "sm100_ptx.cuh"
 
 namespace mpcl {
 
@@ -31,8 +44,12 @@ constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
 constexpr int BM_SMALL = 16;     // tile rows of the small-grid variant
 constexpr int GV_M = 8;         // rows handled by the skinny kernel
 constexpr int GV_KC = 128;      // K chunk staged in shared memory
-constexpr int GV_NARROW = 256;  // widest layer (N) on the narrow GEMV (measured: faster up to N = 128-256,
-                                // slower when streaming 4096-wide rows)
+constexpr int PORTABLE_CLUSTER = 8, MAX_CLUSTER = 16;
+constexpr int GV_NARROW = 256;  // N up to here: ring_gemv_kernel for any K
+constexpr int GV_GRID = 200;    // blocks up to which wider layers take it too, when their K splits fit one
+                                // cluster (measured: 4 x 512 x 1000, 128 blocks, 11.5 -> 9.1 us; 1 x 512 x 4096,
+                                // 512 blocks, would go from 6.7 to 9.4)
+
 
 // element kv of row m of the left operand [E | X + cE] (one_half: X + cE)
 template <int W>
@@ -54,13 +71,58 @@ __device__ __forceinline__ typename Elem<W>::T coef_value(const GemmArgs& a) {
     return 0;
 }
 
-template <int W, int TM>
+// The blocks of a cluster (all of grid.z of one output tile, or a group of it)
+// have written their sums of the same `count` outputs to `part` in their own
+// shared memory: block r adds up one contiguous share of the outputs over the
+// cluster and passes each sum to out(index, sum).
+template <int W, typename Out>
+__device__ __forceinline__ void cluster_sums(const typename Elem<W>::T* part, int count, Out out) {
+    using T = typename Elem<W>::T;
+    const int cs = (int)ptx::cluster_size(), rank = (int)ptx::cluster_rank();
+    __syncwarp();
+    ptx::cluster_sync();        // every block's sums are written
+    const int per = (count + cs - 1) / cs;
+    const int end = min(count, (rank + 1) * per);
+    for (int i = rank * per + (int)threadIdx.x; i < end; i += NT) {
+        T s = 0;
+#pragma unroll 4
+        for (int r = 0; r < cs; ++r) {
+            const uint32_t at = ptx::cluster_addr(part + i, (uint32_t)r);
+            if constexpr (W == 1) {
+                s += ptx::ld_cluster_u64(at);
+            } else {
+                s += (T)ptx::ld_cluster_u64(at) | ((T)ptx::ld_cluster_u64(at + 8) << 64);
+            }
+        }
+        out(i, s);
+    }
+    __syncwarp();
+    ptx::cluster_sync();        // and read, before a block leaves
+}
+
+// Z = C + sum, or Z += sum where several clusters share the output
+template <int W>
+__device__ __forceinline__ void put(const GemmArgs& a, int64_t e, typename Elem<W>::T v, int atomic) {
+    using T = typename Elem<W>::T;
+    if (atomic) atomic_add_elem<W>(a.Z, e, v);
+    else st_elem<W>(a.Z, e, (a.C ? ldg_elem<W>(a.C, e) : (T)0) + v);
+}
+
+// The operands of the next K slice are loaded while the present one is
+// multiplied; not in 16-row Z_2^128 tiles of more than 16 columns, which are
+// bound by their wide multiply-adds (300 x 300 x 300: 84.6 us with it, 82.5
+// without).  CLUSTER: the K splits of a tile are the blocks of a cluster.
+template <int W, int TM, bool CLUSTER, int J>
 __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t kchunk, int atomic) {
     using T = typename Elem<W>::T;
     constexpr int RI = TM / 16;        // rows of a thread's sub-tile
+    constexpr int LV = TM * BK / NT, RV = BK * BN / NT;     // values a thread stages
     __shared__ T Ls[BK][TM + 1];
-    __shared__ T Rs[BK][BN];
+    __shared__ T Rs[BK][BN];           // at the end, the sums of a 16-row tile
+    static_assert(!CLUSTER || TM <= BK, "the sums fit the staged right operand");
 
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;
     const int64_t m0 = (int64_t)blockIdx.y * TM, n0 = (int64_t)blockIdx.x * BN;
@@ -76,51 +138,79 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0;
 
-    for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
-#pragma unroll
-        for (int r = 0; r < (TM * BK) / NT; ++r) {
-            int idx = tid + r * NT;
-            int mm = idx / BK, kk = idx % BK;
-            int64_t m = m0 + mm, kv = k0 + kk;
-            Ls[kk][mm] = (m < M && kv < kend) ? left<W>(a, c, m, kv) : (T)0;
-        }
-#pragma unroll
-        for (int r = 0; r < (BK * BN) / NT; ++r) {
-            int idx = tid + r * NT;
-            int kk = idx / BN, nn = idx % BN;
-            int64_t n = n0 + nn, kv = k0 + kk;
-            T v = 0;
-            if (n < N && kv < kend) {
-                const int64_t kq = kv + kr;
-                v = kq < K ? ldg_elem<W>(a.B, kq * N + n) : ldg_elem<W>(a.F, (kq - K) * N + n);
-            }
-            Rs[kk][nn] = v;
-        }
-        __syncthreads();
+    auto left_at = [&](int idx, int64_t k0) {
+        const int64_t m = m0 + idx / BK, kv = k0 + idx % BK;
+        return (m < M && kv < kend) ? left<W>(a, c, m, kv) : (T)0;
+    };
+    auto right_at = [&](int idx, int64_t k0) {
+        const int64_t n = n0 + idx % BN, kv = k0 + idx / BN;
+        if (n >= N || kv >= kend) return (T)0;
+        const int64_t kq = kv + kr;
+        return kq < K ? ldg_elem<W>(a.B, kq * N + n) : ldg_elem<W>(a.F, (kq - K) * N + n);
+    };
+    auto multiply = [&] {
 #pragma unroll 4
         for (int kk = 0; kk < BK; ++kk) {
-            T av[RI], bv[4];
+            T av[RI], bv[J];
 #pragma unroll
             for (int i = 0; i < RI; ++i) av[i] = Ls[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bv[j] = Rs[kk][tx + 16 * j];
+            for (int j = 0; j < J; ++j) bv[j] = Rs[kk][tx + 16 * j];
 #pragma unroll
             for (int i = 0; i < RI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * bv[j];
+                for (int j = 0; j < J; ++j) acc[i][j] += av[i] * bv[j];
         }
-        __syncthreads();
+    };
+    if constexpr (W == 1 || TM == BM || J == 1 || CLUSTER) {
+        T lv[LV], rv[RV];
+        auto fetch = [&](int64_t k0) {
+#pragma unroll
+            for (int r = 0; r < LV; ++r) lv[r] = left_at(tid + r * NT, k0);
+#pragma unroll
+            for (int r = 0; r < RV; ++r) rv[r] = right_at(tid + r * NT, k0);
+        };
+        if (kbeg < kend) fetch(kbeg);
+        for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+            for (int r = 0; r < LV; ++r) Ls[(tid + r * NT) % BK][(tid + r * NT) / BK] = lv[r];
+#pragma unroll
+            for (int r = 0; r < RV; ++r) Rs[(tid + r * NT) / BN][(tid + r * NT) % BN] = rv[r];
+            __syncthreads();
+            if (k0 + BK < kend) fetch(k0 + BK);
+            multiply();
+            __syncthreads();
+        }
+    } else {
+        for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+            for (int r = 0; r < LV; ++r)
+                Ls[(tid + r * NT) % BK][(tid + r * NT) / BK] = left_at(tid + r * NT, k0);
+#pragma unroll
+            for (int r = 0; r < RV; ++r)
+                Rs[(tid + r * NT) / BN][(tid + r * NT) % BN] = right_at(tid + r * NT, k0);
+            __syncthreads();
+            multiply();
+            __syncthreads();
+        }
     }
+    if constexpr (CLUSTER) {
 #pragma unroll
-    for (int i = 0; i < RI; ++i) {
-        int64_t m = m0 + ty + 16 * i;
-        if (m >= M) continue;
+        for (int j = 0; j < 4; ++j) Rs[ty][tx + 16 * j] = acc[0][j];
+        cluster_sums<W>(&Rs[0][0], BM_SMALL * BN, [&](int i, T v) {
+            const int64_t m = m0 + i / BN, n = n0 + i % BN;
+            if (m < M && n < N) put<W>(a, m * N + n, v, 0);
+        });
+    } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            int64_t n = n0 + tx + 16 * j;
-            if (n >= N) continue;
-            if (atomic) atomic_add_elem<W>(a.Z, m * N + n, acc[i][j]);
-            else st_elem<W>(a.Z, m * N + n, (a.C ? ldg_elem<W>(a.C, m * N + n) : (T)0) + acc[i][j]);
+        for (int i = 0; i < RI; ++i) {
+            int64_t m = m0 + ty + 16 * i;
+            if (m >= M) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                int64_t n = n0 + tx + 16 * j;
+                if (n < N) put<W>(a, m * N + n, acc[i][j], atomic);
+            }
         }
     }
 }
@@ -130,9 +220,11 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
 // two adjacent Z_2^64 columns per thread, read as one 16-byte vector (needs
 // even N); VEC = 1 otherwise.  MM >= M rows are accumulated (1, 2, 4 or 8).
 template <int W, int VEC, int MM>
-__global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchunk, int atomic) {
+__global__ void __launch_bounds__(NT) ring_gemv_wide_kernel(GemmArgs a, int64_t kchunk, int atomic) {
     using T = typename Elem<W>::T;
     __shared__ T Ls[MM][GV_KC];
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int64_t n = ((int64_t)blockIdx.x * NT + threadIdx.x) * VEC;
     const int64_t K = a.K, N = a.N, K2 = a.one_half ? a.K : 2 * a.K;
     const int64_t kr = a.one_half ? K : 0;   // row offset into [B ; F]
@@ -174,31 +266,27 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
         __syncthreads();
     }
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) {
-        const int64_t col = n + v;
-        if (col >= N) break;
+    for (int v = 0; v < VEC; ++v)
 #pragma unroll
-        for (int i = 0; i < MM; ++i) {
-            if (i >= M) break;
-            if (atomic) atomic_add_elem<W>(a.Z, (int64_t)i * N + col, acc[i][v]);
-            else st_elem<W>(a.Z, (int64_t)i * N + col,
-                            (a.C ? ldg_elem<W>(a.C, (int64_t)i * N + col) : (T)0) + acc[i][v]);
-        }
-    }
+        for (int i = 0; i < MM; ++i)
+            if (i < M && n + v < N) put<W>(a, (int64_t)i * N + n + v, acc[i][v], atomic);
 }
 
-// GEMV for narrow layers (N <= GV_NARROW): a block covers 32 lanes x VEC
-// output columns and its eight warps take rows w, w + 8, ... of each staged K
-// chunk; the warps' sums are added in shared memory before the block writes
-// (or atomically adds) one partial per output, so that many blocks can share
-// the K range of few columns.  VEC and MM as above.
+// GEMV (M <= GV_M): a block covers 32 lanes x VEC output columns (VEC = 2: two
+// adjacent Z_2^64 columns as one 16-byte vector, which needs even N) and its
+// eight warps take rows w, w + 8, ... of each staged K chunk; MM >= M rows are
+// accumulated (1, 2, 4 or 8).  The warps' sums are added in shared memory and
+// the cluster's blocks, which split K, add theirs through distributed shared
+// memory.
 template <int W, int VEC, int MM>
-__global__ void __launch_bounds__(NT) ring_gemv_narrow_kernel(GemmArgs a, int64_t kchunk, int atomic) {
+__global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchunk, int atomic) {
     using T = typename Elem<W>::T;
     constexpr int NW = NT / 32;                 // warps per block
     constexpr int NCOL = 32 * VEC;              // columns per block
     __shared__ T Ls[MM][GV_KC];
     __shared__ T red[NW - 1][MM][NCOL];         // sums of warps 1 .. NW - 1
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n = (int64_t)blockIdx.x * NCOL + lane * VEC;
     const int64_t K = a.K, N = a.N, K2 = a.one_half ? a.K : 2 * a.K;
@@ -220,7 +308,7 @@ __global__ void __launch_bounds__(NT) ring_gemv_narrow_kernel(GemmArgs a, int64_
         }
         __syncthreads();
         if (n < N) {
-#pragma unroll 4
+#pragma unroll 8
             for (int kk = warp; kk < kc; kk += NW) {
                 const int64_t kv = k0 + kk + kr;
                 const u64* row = kv < K ? a.B + kv * N * W : a.F + (kv - K) * N * W;
@@ -247,25 +335,33 @@ __global__ void __launch_bounds__(NT) ring_gemv_narrow_kernel(GemmArgs a, int64_
             for (int v = 0; v < VEC; ++v) red[warp - 1][i][lane * VEC + v] = acc[i][v];
     }
     __syncthreads();
-    if (warp != 0) return;
+    T* part = &Ls[0][0];                        // every warp is done with the staged rows
+    if (warp == 0) {
 #pragma unroll
-    for (int w = 0; w < NW - 1; ++w)
+        for (int w = 0; w < NW - 1; ++w)
 #pragma unroll
-        for (int i = 0; i < MM; ++i)
+            for (int i = 0; i < MM; ++i)
 #pragma unroll
-            for (int v = 0; v < VEC; ++v) acc[i][v] += red[w][i][lane * VEC + v];
+                for (int v = 0; v < VEC; ++v) acc[i][v] += red[w][i][lane * VEC + v];
+        if (ptx::cluster_size() == 1) {
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) {
-        const int64_t col = n + v;
-        if (col >= N) break;
+            for (int i = 0; i < MM; ++i)
 #pragma unroll
-        for (int i = 0; i < MM; ++i) {
-            if (i >= M) break;
-            if (atomic) atomic_add_elem<W>(a.Z, (int64_t)i * N + col, acc[i][v]);
-            else st_elem<W>(a.Z, (int64_t)i * N + col,
-                            (a.C ? ldg_elem<W>(a.C, (int64_t)i * N + col) : (T)0) + acc[i][v]);
+                for (int v = 0; v < VEC; ++v)
+                    if (i < M && n + v < N) put<W>(a, (int64_t)i * N + n + v, acc[i][v], atomic);
+        } else {
+#pragma unroll
+            for (int i = 0; i < MM; ++i)
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) part[i * NCOL + lane * VEC + v] = acc[i][v];
         }
     }
+    if (ptx::cluster_size() == 1) return;
+    cluster_sums<W>(part, MM * NCOL, [&](int i, T v) {
+        const int row = i / NCOL;
+        const int64_t col = (int64_t)blockIdx.x * NCOL + i % NCOL;
+        if (row < M && col < N) put<W>(a, row * N + col, v, atomic);
+    });
 }
 
 // K chunks (multiples of `step`, at least `min_chunk`) so that the grid covers
@@ -291,58 +387,101 @@ int simt_tile_rows(int64_t M, int64_t N, int rows) {
 
 namespace {
 
+using Kernel = void (*)(GemmArgs, int64_t, int);
+
+template <int W, int J> Kernel tile_kernel(int tm, bool cluster) {
+    if (tm == BM) return ring_gemm_simt_kernel<W, BM, false, J>;
+    return cluster ? ring_gemm_simt_kernel<W, BM_SMALL, true, J> : ring_gemm_simt_kernel<W, BM_SMALL, false, J>;
+}
+
+template <int W, int VEC> Kernel gemv_kernel(int64_t M, bool wide) {
+    if (wide)
+        return M <= 1   ? ring_gemv_wide_kernel<W, VEC, 1>
+               : M <= 2 ? ring_gemv_wide_kernel<W, VEC, 2>
+               : M <= 4 ? ring_gemv_wide_kernel<W, VEC, 4>
+                        : ring_gemv_wide_kernel<W, VEC, 8>;
+    return M <= 1   ? ring_gemv_kernel<W, VEC, 1>
+           : M <= 2 ? ring_gemv_kernel<W, VEC, 2>
+           : M <= 4 ? ring_gemv_kernel<W, VEC, 4>
+                    : ring_gemv_kernel<W, VEC, 8>;
+}
+
 template <int W>
-cudaError_t run(const GemmArgs& a, cudaStream_t st) {
+cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
     const int64_t K2 = a.one_half ? a.K : 2 * a.K;
     const bool skinny = a.M <= GV_M;
     const int vec = (skinny && W == 1 && a.N % 2 == 0) ? 2 : 1;
     const int tm = simt_tile_rows(a.M, a.N, a.rows);
-    const bool narrow = skinny && a.N <= GV_NARROW;
-    const int64_t cols = narrow ? 32 * vec : NT * vec;   // columns per GEMV block
-    const int64_t bx = skinny ? (a.N + cols - 1) / cols : (a.N + BN - 1) / BN;
     const int64_t by = skinny ? 1 : (a.M + tm - 1) / tm;
     if (by > 65535) return cudaErrorInvalidConfiguration;
-    // K split so that the grid covers about `waves` x 152 blocks (launch table, else 4 / 2);
-    // GEMV chunks give each of a block's eight warps at least 16 rows
     const int64_t waves = a.simt_waves > 0 ? a.simt_waves : (skinny ? 4 : 2);
-    const int64_t kchunk = skinny ? choose_kchunk(bx * by, K2, 16, narrow ? 128 : 32, waves)
-                                  : choose_kchunk(bx * by, K2, BK, 4 * BK, waves);
-    const int64_t bz = K2 > 0 ? (K2 + kchunk - 1) / kchunk : 1;
+    int64_t bx = skinny ? (a.N + 32 * vec - 1) / (32 * vec) : (a.N + BN - 1) / BN;
+    // one cluster per output tile with all of its K splits, where that gives
+    // blocks little work: no atomics, and no pass to set Z to C before them
+    const int64_t least = skinny ? 128 : BK;         // K of a block, at least
+    int64_t splits = (K2 + least - 1) / least;
+    if (skinny && a.N <= GV_NARROW) splits = std::min(splits, std::max<int64_t>(1, waves * 152 / bx));
+    int cs = 1;
+    while (cs < splits && cs < MAX_CLUSTER) cs *= 2;
+    if (!skinny)
+        while (cs > 1 && bx * by * cs > 152) cs /= 2;
+    const bool cluster = skinny ? cs >= splits && (a.N <= GV_NARROW || bx * cs <= GV_GRID)
+                                // 48 (16): beyond three (one) slices per block more splits with
+                                // atomics are faster: 16 x 400 x 160 in Z_2^64 9.9 us as clusters, 8.5 so
+                                : tm == BM_SMALL && cs > 1 && K2 <= cs * (W == 1 ? 48 : 16);
+    const bool wide = skinny && a.N > GV_NARROW && !cluster;
+    int64_t kchunk, bz;
+    if (cluster) {
+        bz = cs;
+        kchunk = ((K2 + bz - 1) / bz + 15) / 16 * 16;
+    } else {
+        // the grid covers about `waves` x 152 blocks (launch table, else 4 / 2); GEMV chunks
+        // give each of a block's eight warps at least 16 rows
+        cs = 1;
+        if (wide) bx = (a.N + NT * vec - 1) / (NT * vec);
+        kchunk = choose_kchunk(bx * by, K2, 16, wide ? 32 : skinny ? 128 : 4 * BK, waves);
+        bz = K2 > 0 ? (K2 + kchunk - 1) / kchunk : 1;
+    }
     if (bz > 65535) return cudaErrorInvalidConfiguration;
-    const int atomic = bz > 1 ? 1 : 0;
+    const int atomic = bz > cs ? 1 : 0;
     if (atomic) {
         const size_t bytes = (size_t)a.M * a.N * 8 * W;
         cudaError_t e = a.C ? cudaMemcpyAsync(a.Z, a.C, bytes, cudaMemcpyDeviceToDevice, st)
                             : cudaMemsetAsync(a.Z, 0, bytes, st);
         if (e != cudaSuccess) return e;
     }
-    dim3 grid((unsigned)bx, (unsigned)by, (unsigned)bz);
-    if (skinny) {
-        const int mm = a.M <= 1 ? 1 : a.M <= 2 ? 2 : a.M <= 4 ? 4 : 8;
-#define MPCL_GEMV(V, R)                                                                  \
-    (narrow ? ring_gemv_narrow_kernel<W, V, R><<<grid, NT, 0, st>>>(a, kchunk, atomic)   \
-            : ring_gemv_kernel<W, V, R><<<grid, NT, 0, st>>>(a, kchunk, atomic))
-        if (vec == 2) {
-            if (mm == 1) MPCL_GEMV(2, 1); else if (mm == 2) MPCL_GEMV(2, 2);
-            else if (mm == 4) MPCL_GEMV(2, 4); else MPCL_GEMV(2, 8);
-        } else {
-            if (mm == 1) MPCL_GEMV(1, 1); else if (mm == 2) MPCL_GEMV(1, 2);
-            else if (mm == 4) MPCL_GEMV(1, 4); else MPCL_GEMV(1, 8);
-        }
-#undef MPCL_GEMV
-    } else if (tm == BM_SMALL) {
-        ring_gemm_simt_kernel<W, BM_SMALL><<<grid, NT, 0, st>>>(a, kchunk, atomic);
-    } else {
-        ring_gemm_simt_kernel<W, BM><<<grid, NT, 0, st>>>(a, kchunk, atomic);
+    const dim3 grid((unsigned)bx, (unsigned)by, (unsigned)bz);
+    const Kernel kernel = !skinny     ? (a.N <= 16 ? tile_kernel<W, 1>(tm, cluster) : tile_kernel<W, 4>(tm, cluster))
+                          : vec == 2 ? gemv_kernel<W, 3 - W>(a.M, wide)
+                                     : gemv_kernel<W, 1>(a.M, wide);
+    if (cs > PORTABLE_CLUSTER) {
+        const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NT);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (dependent) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cs > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = 1;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = (unsigned)cs;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, a, kchunk, atomic);
 }
 
 }  // namespace
 
-cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t st) {
+cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t st, bool dependent) {
     if (a.M == 0 || a.N == 0) return cudaSuccess;
-    return a.words == 1 ? run<1>(a, st) : run<2>(a, st);
+    return a.words == 1 ? run<1>(a, st, dependent) : run<2>(a, st, dependent);
 }
 
 }  // namespace mpcl

@@ -55,7 +55,8 @@ constexpr int TALL_TILE_ROWS = -128;
 // the launch-table value of the residue path (gemm_crt.cu: 256 x 256 tiles)
 constexpr int CRT_TILE_ROWS = 256;
 
-cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t st);
+// dependent: launched as a dependent of the kernel before it in the stream
+cudaError_t launch_gemm_simt(const GemmArgs& a, cudaStream_t st, bool dependent);
 
 // tensor-core ring GEMM (fp16 digit products, exact); returns
 // cudaErrorNotSupported when the shape is not handled by it.

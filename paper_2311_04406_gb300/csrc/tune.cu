@@ -120,7 +120,7 @@ float time_candidate(const mpcl::GemmArgs& a, const mpcl::Choice& c, void* ws, s
     g.rows = c.rows;
     auto run = [&]() -> cudaError_t {
         if (c.path == 1 && c.rows == mpcl::CRT_TILE_ROWS) return mpcl::launch_gemm_crt(g, ws, ws_bytes, st);
-        return c.path == 1 ? mpcl::launch_gemm_tc(g, ws, ws_bytes, st) : mpcl::launch_gemm_simt(g, st);
+        return c.path == 1 ? mpcl::launch_gemm_tc(g, ws, ws_bytes, st) : mpcl::launch_gemm_simt(g, st, true);
     };
     *ok = false;
     if (run() != cudaSuccess) return 0.f;
