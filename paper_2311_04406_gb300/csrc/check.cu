@@ -96,17 +96,42 @@ __global__ void __launch_bounds__(NT) check_compact_group_kernel(const __grid_co
     check_compact<W>(g.M[l], g.alpha[l], g.chi_hat[l], g.Dc[l], g.mDc[l], g.cs[l]);
 }
 
+// f(i, W_i, m(W)_i) for this thread's elements, the loads of four in flight
+// together.  (With one at a time and a launch gap before each of the kernels, the
+// masks, opening and check of 2047 x 1025 values in Z_2^128 took 126 us; now 112,
+// of which 104 are their 704 MB.)
+template <int W, typename F>
+__device__ __forceinline__ void sweep(int64_t n, const u64* Wm, const u64* mW, F f) {
+    using T = typename Elem<W>::T;
+    constexpr int U = 4;
+    const int64_t step = (int64_t)gridDim.x * NT;
+    int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x;
+    for (; i + (U - 1) * step < n; i += U * step) {
+        T w[U], m[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            w[j] = ldg_elem<W>(Wm, i + j * step);
+            m[j] = ldg_elem<W>(mW, i + j * step);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) f(i + j * step, w[j], m[j]);
+    }
+    for (; i < n; i += step) f(i, ldg_elem<W>(Wm, i), ldg_elem<W>(mW, i));
+}
+
 template <int W>
 __global__ void __launch_bounds__(NT) batchrec_partial_kernel(int64_t n, const u64* alpha,
                                                               const u64* chi, const u64* Wm,
                                                               const u64* mW, u64* part) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     const T a = ld_elem<W>(alpha, 0);
     T acc = 0;
-    for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
-        T x = ldg_elem<W>(chi, i);
-        acc += ldg_elem<W>(mW, i) * x - a * (ldg_elem<W>(Wm, i) * x);
-    }
+    sweep<W>(n, Wm, mW, [&](int64_t i, T w, T m) {
+        const T x = ldg_elem<W>(chi, i);
+        acc += m * x - a * (w * x);
+    });
     T tot = block_sum<W>(acc);
     if (threadIdx.x == 0) st_elem<W>(part, blockIdx.x, tot);
 }
@@ -125,15 +150,17 @@ template <int W>
 __global__ void __launch_bounds__(NT) batchrec_seeded_partial_kernel(int64_t n, int s, const u64* alpha,
                                                                      const u64* seedp, const u64* Wm,
                                                                      const u64* mW, u64* part) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     const T a = ld_elem<W>(alpha, 0);
     const u64 seed = seedp[0];
     const u64 ms = s >= 64 ? ~0ull : ((1ull << s) - 1);
     T acc = 0;
-    for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
+    sweep<W>(n, Wm, mW, [&](int64_t i, T w, T m) {
         const T x = (T)(splitmix64_at(seed, i) & ms);
-        acc += ldg_elem<W>(mW, i) * x - a * (ldg_elem<W>(Wm, i) * x);
-    }
+        acc += m * x - a * (w * x);
+    });
     T tot = block_sum<W>(acc);
     if (threadIdx.x == 0) st_elem<W>(part, blockIdx.x, tot);
 }
@@ -144,6 +171,8 @@ template <int W>
 __global__ void __launch_bounds__(NT) batchrec_mask_kernel(int64_t n, const u64* X, const u64* A,
                                                            const u64* R, const u64* mX, const u64* mA,
                                                            const u64* mR, u64* Wo, u64* mWo) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
         T v = ldg_elem<W>(X, i) + ldg_elem<W>(R, i);
@@ -157,6 +186,8 @@ __global__ void __launch_bounds__(NT) batchrec_mask_kernel(int64_t n, const u64*
 
 template <int W>
 __global__ void __launch_bounds__(NT) sum_kernel(int64_t n, const u64* part, u64* out) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     T acc = 0;
     for (int64_t i = threadIdx.x; i < n; i += NT) acc += ld_elem<W>(part, i);
@@ -212,13 +243,11 @@ cudaError_t launch_check_batchrec_seeded(int64_t M, int64_t N, int words, int s,
     const int64_t blocks = batchrec_blocks(n);
     if (ws_bytes < (size_t)blocks * 8 * (size_t)words) return cudaErrorInvalidValue;
     u64* part = (u64*)ws;
-    if (words == 1) {
-        batchrec_seeded_partial_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(n, s, alpha, seed, Wm, mW, part);
-        sum_kernel<1><<<1, NT, 0, st>>>(blocks, part, cs);
-    } else {
-        batchrec_seeded_partial_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(n, s, alpha, seed, Wm, mW, part);
-        sum_kernel<2><<<1, NT, 0, st>>>(blocks, part, cs);
-    }
+    cudaError_t e = launch_dependent(words == 1 ? batchrec_seeded_partial_kernel<1> : batchrec_seeded_partial_kernel<2>,
+                                     dim3((unsigned)blocks), dim3(NT), 0, st, n, s, alpha, seed, Wm, mW, part);
+    if (e == cudaSuccess)
+        e = launch_dependent(words == 1 ? sum_kernel<1> : sum_kernel<2>, dim3(1), dim3(NT), 0, st, blocks, part, cs);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -228,8 +257,9 @@ cudaError_t launch_batchrec_mask(int64_t n, int words, const u64* X, const u64* 
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + NT - 1) / NT;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    if (words == 1) batchrec_mask_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(n, X, A, R, mX, mA, mR, Wo, mWo);
-    else batchrec_mask_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(n, X, A, R, mX, mA, mR, Wo, mWo);
+    const cudaError_t e = launch_dependent(words == 1 ? batchrec_mask_kernel<1> : batchrec_mask_kernel<2>,
+                                           dim3((unsigned)blocks), dim3(NT), 0, st, n, X, A, R, mX, mA, mR, Wo, mWo);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -244,13 +274,11 @@ cudaError_t launch_check_batchrec(int64_t M, int64_t N, int words, const u64* al
     const int64_t blocks = batchrec_blocks(n);
     if (ws_bytes < check_batchrec_workspace(M, N, words)) return cudaErrorInvalidValue;
     u64* part = (u64*)ws;
-    if (words == 1) {
-        batchrec_partial_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(n, alpha, chi, Wm, mW, part);
-        sum_kernel<1><<<1, NT, 0, st>>>(blocks, part, cs);
-    } else {
-        batchrec_partial_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(n, alpha, chi, Wm, mW, part);
-        sum_kernel<2><<<1, NT, 0, st>>>(blocks, part, cs);
-    }
+    cudaError_t e = launch_dependent(words == 1 ? batchrec_partial_kernel<1> : batchrec_partial_kernel<2>,
+                                     dim3((unsigned)blocks), dim3(NT), 0, st, n, alpha, chi, Wm, mW, part);
+    if (e == cudaSuccess)
+        e = launch_dependent(words == 1 ? sum_kernel<1> : sum_kernel<2>, dim3(1), dim3(NT), 0, st, blocks, part, cs);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 

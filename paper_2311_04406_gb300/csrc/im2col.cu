@@ -6,6 +6,7 @@
 // (§2.4), so each party applies this to its own shares and tags locally.
 #include "common.cuh"
 #include "kernels.h"
+#include "sm100_ptx.cuh"
 
 namespace mpcl {
 
@@ -36,6 +37,8 @@ constexpr int UNROLL = 4;       // loads in flight per thread
 template <int WW>
 __global__ void __launch_bounds__(NT) im2col_kernel(const Im2colArgs a, uint32_t rows, uint32_t Kc, uint32_t tx,
                                                     uint32_t col_blocks, uint32_t run) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<WW>::T;
     const uint32_t rb = blockIdx.x / col_blocks;
     const uint32_t col = (blockIdx.x - rb * col_blocks) * tx + (threadIdx.x & (tx - 1));
@@ -91,10 +94,8 @@ cudaError_t launch_im2col(int64_t B, int64_t C, int64_t H, int64_t W, int f, int
     const int64_t passes = (rows + step * UNROLL - 1) / (step * UNROLL);
     const int64_t per = (passes * col_blocks + BLOCKS - 1) / BLOCKS;
     const int64_t run = per * step * UNROLL, blocks = (rows + run - 1) / run * col_blocks;
-    auto* kernel = words == 1 ? im2col_kernel<1> : im2col_kernel<2>;
-    kernel<<<(unsigned)blocks, NT, 0, st>>>(a, (uint32_t)rows, (uint32_t)Kc, (uint32_t)tx, (uint32_t)col_blocks,
-                                            (uint32_t)run);
-    return cudaGetLastError();
+    return launch_dependent(words == 1 ? im2col_kernel<1> : im2col_kernel<2>, dim3((unsigned)blocks), dim3(NT), 0, st, a,
+                            (uint32_t)rows, (uint32_t)Kc, (uint32_t)tx, (uint32_t)col_blocks, (uint32_t)run);
 }
 
 }  // namespace mpcl

@@ -5,6 +5,7 @@
 // (linearity of authenticated shares under public constants, §2.4).
 #include "common.cuh"
 #include "kernels.h"
+#include "sm100_ptx.cuh"
 
 namespace mpcl {
 
@@ -22,6 +23,8 @@ struct LincombArgs {
 
 template <int W>
 __global__ void __launch_bounds__(NT) lincomb_kernel(const __grid_constant__ LincombArgs a) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     if constexpr (W == 1) {
         // two elements per 16-byte access when n is even (else one at a time)
@@ -68,6 +71,8 @@ constexpr int GROUP_ELEMS = NT * 4;   // elements per block of a grouped launch
 
 template <int W>
 __global__ void __launch_bounds__(NT) lincomb_group_kernel(const __grid_constant__ LincombGroup a) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     int lo = 0, hi = a.groups - 1;
     while (lo < hi) {
@@ -109,9 +114,8 @@ cudaError_t launch_lincomb_grouped(int groups, const int64_t* n, int words, int 
         a.groups = k;
         const int64_t blocks = a.b_off[k];
         if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-        if (words == 1) lincomb_group_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(a);
-        else lincomb_group_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(a);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_dependent(words == 1 ? lincomb_group_kernel<1> : lincomb_group_kernel<2>,
+                                               dim3((unsigned)blocks), dim3(NT), 0, st, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -133,9 +137,8 @@ cudaError_t launch_lincomb(int64_t n, int words, int count, const int64_t* coef,
     int64_t blocks = (n / per + NT - 1) / NT;
     if (blocks > 152 * 16) blocks = 152 * 16;
     if (blocks < 1) blocks = 1;
-    if (words == 1) lincomb_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(a);
-    else lincomb_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(words == 1 ? lincomb_kernel<1> : lincomb_kernel<2>, dim3((unsigned)blocks), dim3(NT), 0,
+                            st, a);
 }
 
 }  // namespace mpcl

@@ -7,6 +7,7 @@
 // conflicts) keep both the reads and the writes coalesced.
 #include "common.cuh"
 #include "kernels.h"
+#include "sm100_ptx.cuh"
 
 namespace mpcl {
 
@@ -17,6 +18,8 @@ constexpr int TILE = 32, ROWS = 8;
 template <int W>
 __global__ void __launch_bounds__(TILE * ROWS) transpose_kernel(int64_t rows, int64_t cols, const u64* in,
                                                                 u64* out) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     __shared__ T tile[TILE][TILE + 1];
     const int64_t c0 = (int64_t)blockIdx.x * TILE, r0 = (int64_t)blockIdx.y * TILE;
@@ -42,9 +45,8 @@ cudaError_t launch_transpose(int64_t rows, int64_t cols, int words, const u64* i
     const int64_t gx = (cols + TILE - 1) / TILE, gy = (rows + TILE - 1) / TILE;
     if (gy > 65535) return cudaErrorInvalidConfiguration;
     dim3 grid((unsigned)gx, (unsigned)gy), block(TILE, ROWS);
-    if (words == 1) transpose_kernel<1><<<grid, block, 0, st>>>(rows, cols, in, out);
-    else transpose_kernel<2><<<grid, block, 0, st>>>(rows, cols, in, out);
-    return cudaGetLastError();
+    return launch_dependent(words == 1 ? transpose_kernel<1> : transpose_kernel<2>, grid, block, 0, st, rows, cols, in,
+                            out);
 }
 
 }  // namespace mpcl

@@ -7,6 +7,7 @@
 // "/ 2^f" is the floor division of the k-bit value; all sums wrap mod 2^(k+s).
 #include "common.cuh"
 #include "kernels.h"
+#include "sm100_ptx.cuh"
 
 namespace mpcl {
 
@@ -19,6 +20,8 @@ __global__ void __launch_bounds__(NT) optmac_trunc_kernel(int64_t MN, int k, int
                                                           const u64* alpha, const u64* Rf,
                                                           const u64* mRf, const u64* Dt, const u64* P,
                                                           u64* Zf, u64* mZf) {
+    ptx::grid_dep_launch();
+    ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     const T mk = k >= 64 * W ? ~(T)0 : (((T)1 << k) - 1);
     const T a = ld_elem<W>(alpha, 0);
@@ -39,11 +42,8 @@ cudaError_t launch_optmac_trunc(int64_t MN, int words, int k, int f, int party0,
     if (MN == 0) return cudaSuccess;
     int64_t blocks = (MN + NT - 1) / NT;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    if (words == 1)
-        optmac_trunc_kernel<1><<<(unsigned)blocks, NT, 0, st>>>(MN, k, f, party0, alpha, Rf, mRf, Dt, P, Zf, mZf);
-    else
-        optmac_trunc_kernel<2><<<(unsigned)blocks, NT, 0, st>>>(MN, k, f, party0, alpha, Rf, mRf, Dt, P, Zf, mZf);
-    return cudaGetLastError();
+    return launch_dependent(words == 1 ? optmac_trunc_kernel<1> : optmac_trunc_kernel<2>, dim3((unsigned)blocks),
+                            dim3(NT), 0, st, MN, k, f, party0, alpha, Rf, mRf, Dt, P, Zf, mZf);
 }
 
 }  // namespace mpcl
