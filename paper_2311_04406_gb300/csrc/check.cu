@@ -41,30 +41,51 @@ __device__ typename Elem<W>::T block_sum(typename Elem<W>::T v) {
     return tot;  // valid in thread 0
 }
 
-// The check sum of one layer by one block.  Bound by the latency of its loads:
-// four rows per thread are loaded together (32,768 rows took 37 us with one).
+// The check sum of one layer by the blocks of a cluster, which share out its
+// rows; the block of rank 0 adds up their sums.  Bound by the latency of its
+// loads: four rows per thread are loaded together (32,768 rows took 37 us with
+// one), and layers of more than CHECK_ROWS rows take eight blocks (the checks of
+// VGG-16 at batch 32 took 28 us with one; the whole pass got 24 us shorter).
+constexpr int64_t CHECK_ROWS = 4 * NT;
+constexpr int CHECK_CLUSTER = 8;
 template <int W>
 __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const u64* chi_hat, const u64* Dc,
                                               const u64* mDc, u64* cs) {
     using T = typename Elem<W>::T;
     constexpr int U = 4;
+    __shared__ T part;
+    const int blocks = (int)ptx::cluster_size(), rank = (int)ptx::cluster_rank();
     const T a = ld_elem<W>(alpha, 0);
     T acc = 0;
-    int64_t r = threadIdx.x;
-    for (; r + (U - 1) * NT < M; r += U * NT) {
+    const int64_t step = (int64_t)blocks * NT;
+    int64_t r = rank * NT + (int)threadIdx.x;
+    for (; r + (U - 1) * step < M; r += U * step) {
         T x[U], d[U], m[U];
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            x[i] = ldg_elem<W>(chi_hat, r + i * NT);
-            d[i] = ldg_elem<W>(Dc, r + i * NT);
-            m[i] = ldg_elem<W>(mDc, r + i * NT);
+            x[i] = ldg_elem<W>(chi_hat, r + i * step);
+            d[i] = ldg_elem<W>(Dc, r + i * step);
+            m[i] = ldg_elem<W>(mDc, r + i * step);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) acc += x[i] * (a * d[i] - m[i]);
     }
-    for (; r < M; r += NT) acc += ldg_elem<W>(chi_hat, r) * (a * ldg_elem<W>(Dc, r) - ldg_elem<W>(mDc, r));
-    const T tot = block_sum<W>(acc);
-    if (threadIdx.x == 0) st_elem<W>(cs, 0, tot);
+    for (; r < M; r += step) acc += ldg_elem<W>(chi_hat, r) * (a * ldg_elem<W>(Dc, r) - ldg_elem<W>(mDc, r));
+    T tot = block_sum<W>(acc);
+    if (blocks > 1) {
+        if (threadIdx.x == 0) part = tot;
+        __syncwarp();
+        ptx::cluster_sync();
+        if (rank == 0 && threadIdx.x == 0)
+            for (int i = 1; i < blocks; ++i) {
+                const uint32_t at = ptx::cluster_addr(&part, (uint32_t)i);
+                if constexpr (W == 1) tot += ptx::ld_cluster_u64(at);
+                else tot += (T)ptx::ld_cluster_u64(at) | ((T)ptx::ld_cluster_u64(at + 8) << 64);
+            }
+        __syncwarp();
+        ptx::cluster_sync();    // the sums are read before a block leaves
+    }
+    if (rank == 0 && threadIdx.x == 0) st_elem<W>(cs, 0, tot);
 }
 
 template <int W>
@@ -76,7 +97,7 @@ __global__ void __launch_bounds__(NT) check_compact_kernel(int64_t M, const u64*
     check_compact<W>(M, alpha, chi_hat, Dc, mDc, cs);
 }
 
-// Up to CHECK_GROUP_MAX compact checks in one launch: block b computes the
+// Up to CHECK_GROUP_MAX compact checks in one launch: cluster b computes the
 // check share of layer b (the same sum as check_compact_kernel).
 struct CheckGroup {
     int count;
@@ -92,7 +113,7 @@ template <int W>
 __global__ void __launch_bounds__(NT) check_compact_group_kernel(const __grid_constant__ CheckGroup g) {
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
-    const int l = blockIdx.x;
+    const int l = blockIdx.x / ptx::cluster_size();
     check_compact<W>(g.M[l], g.alpha[l], g.chi_hat[l], g.Dc[l], g.mDc[l], g.cs[l]);
 }
 
@@ -206,12 +227,9 @@ int64_t batchrec_blocks(int64_t n) {
 
 cudaError_t launch_check_compact(int64_t M, int words, const u64* alpha, const u64* chi_hat,
                                  const u64* Dc, const u64* mDc, u64* cs, cudaStream_t st) {
-    const cudaError_t e = words == 1 ? launch_dependent(check_compact_kernel<1>, dim3(1), dim3(NT), 0, st, M, alpha,
-                                                        chi_hat, Dc, mDc, cs)
-                                     : launch_dependent(check_compact_kernel<2>, dim3(1), dim3(NT), 0, st, M, alpha,
-                                                        chi_hat, Dc, mDc, cs);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    const int blocks = M > CHECK_ROWS ? CHECK_CLUSTER : 1;
+    return launch_dependent_cluster(words == 1 ? check_compact_kernel<1> : check_compact_kernel<2>, dim3(blocks),
+                                    dim3(NT), blocks, st, M, alpha, chi_hat, Dc, mDc, cs);
 }
 
 cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, const u64* const* alpha,
@@ -220,7 +238,9 @@ cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, con
     for (int i0 = 0; i0 < n; i0 += CHECK_GROUP_MAX) {
         CheckGroup g{};
         g.count = n - i0 < CHECK_GROUP_MAX ? n - i0 : CHECK_GROUP_MAX;
+        int blocks = 1;
         for (int j = 0; j < g.count; ++j) {
+            if (M[i0 + j] > CHECK_ROWS) blocks = CHECK_CLUSTER;
             g.M[j] = M[i0 + j];
             g.alpha[j] = alpha[i0 + j];
             g.chi_hat[j] = chi_hat[i0 + j];
@@ -229,11 +249,11 @@ cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, con
             g.cs[j] = cs[i0 + j];
         }
         const cudaError_t e =
-            words == 1 ? launch_dependent(check_compact_group_kernel<1>, dim3(g.count), dim3(NT), 0, st, g)
-                       : launch_dependent(check_compact_group_kernel<2>, dim3(g.count), dim3(NT), 0, st, g);
+            launch_dependent_cluster(words == 1 ? check_compact_group_kernel<1> : check_compact_group_kernel<2>,
+                                     dim3(g.count * blocks), dim3(NT), blocks, st, g);
         if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_check_batchrec_seeded(int64_t M, int64_t N, int words, int s, const u64* alpha,
