@@ -48,13 +48,12 @@ __device__ typename Elem<W>::T block_sum(typename Elem<W>::T v) {
 // VGG-16 at batch 32 took 28 us with one; the whole pass got 24 us shorter).
 constexpr int64_t CHECK_ROWS = 4 * NT;
 constexpr int CHECK_CLUSTER = 8;
-template <int W>
+template <int W, bool CLUSTER>
 __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const u64* chi_hat, const u64* Dc,
                                               const u64* mDc, u64* cs) {
     using T = typename Elem<W>::T;
     constexpr int U = 4;
-    __shared__ T part;
-    const int blocks = (int)ptx::cluster_size(), rank = (int)ptx::cluster_rank();
+    const int blocks = CLUSTER ? CHECK_CLUSTER : 1, rank = CLUSTER ? (int)ptx::cluster_rank() : 0;
     const T a = ld_elem<W>(alpha, 0);
     T acc = 0;
     const int64_t step = (int64_t)blocks * NT;
@@ -72,7 +71,8 @@ __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const
     }
     for (; r < M; r += step) acc += ldg_elem<W>(chi_hat, r) * (a * ldg_elem<W>(Dc, r) - ldg_elem<W>(mDc, r));
     T tot = block_sum<W>(acc);
-    if (blocks > 1) {
+    if constexpr (CLUSTER) {
+        __shared__ T part;
         if (threadIdx.x == 0) part = tot;
         __syncwarp();
         ptx::cluster_sync();
@@ -88,13 +88,13 @@ __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const
     if (rank == 0 && threadIdx.x == 0) st_elem<W>(cs, 0, tot);
 }
 
-template <int W>
+template <int W, bool CLUSTER>
 __global__ void __launch_bounds__(NT) check_compact_kernel(int64_t M, const u64* alpha,
                                                            const u64* chi_hat, const u64* Dc,
                                                            const u64* mDc, u64* cs) {
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
-    check_compact<W>(M, alpha, chi_hat, Dc, mDc, cs);
+    check_compact<W, CLUSTER>(M, alpha, chi_hat, Dc, mDc, cs);
 }
 
 // Up to CHECK_GROUP_MAX compact checks in one launch: cluster b computes the
@@ -109,12 +109,12 @@ struct CheckGroup {
     u64* cs[CHECK_GROUP_MAX];
 };
 
-template <int W>
+template <int W, bool CLUSTER>
 __global__ void __launch_bounds__(NT) check_compact_group_kernel(const __grid_constant__ CheckGroup g) {
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
-    const int l = blockIdx.x / ptx::cluster_size();
-    check_compact<W>(g.M[l], g.alpha[l], g.chi_hat[l], g.Dc[l], g.mDc[l], g.cs[l]);
+    const int l = blockIdx.x / (CLUSTER ? CHECK_CLUSTER : 1);
+    check_compact<W, CLUSTER>(g.M[l], g.alpha[l], g.chi_hat[l], g.Dc[l], g.mDc[l], g.cs[l]);
 }
 
 // f(i, W_i, m(W)_i) for this thread's elements, the loads of four in flight
@@ -227,9 +227,11 @@ int64_t batchrec_blocks(int64_t n) {
 
 cudaError_t launch_check_compact(int64_t M, int words, const u64* alpha, const u64* chi_hat,
                                  const u64* Dc, const u64* mDc, u64* cs, cudaStream_t st) {
-    const int blocks = M > CHECK_ROWS ? CHECK_CLUSTER : 1;
-    return launch_dependent_cluster(words == 1 ? check_compact_kernel<1> : check_compact_kernel<2>, dim3(blocks),
-                                    dim3(NT), blocks, st, M, alpha, chi_hat, Dc, mDc, cs);
+    if (M > CHECK_ROWS)
+        return launch_dependent_cluster(words == 1 ? check_compact_kernel<1, true> : check_compact_kernel<2, true>,
+                                        dim3(CHECK_CLUSTER), dim3(NT), CHECK_CLUSTER, st, M, alpha, chi_hat, Dc, mDc, cs);
+    return launch_dependent(words == 1 ? check_compact_kernel<1, false> : check_compact_kernel<2, false>, dim3(1),
+                            dim3(NT), 0, st, M, alpha, chi_hat, Dc, mDc, cs);
 }
 
 cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, const u64* const* alpha,
@@ -238,9 +240,9 @@ cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, con
     for (int i0 = 0; i0 < n; i0 += CHECK_GROUP_MAX) {
         CheckGroup g{};
         g.count = n - i0 < CHECK_GROUP_MAX ? n - i0 : CHECK_GROUP_MAX;
-        int blocks = 1;
+        bool cluster = false;
         for (int j = 0; j < g.count; ++j) {
-            if (M[i0 + j] > CHECK_ROWS) blocks = CHECK_CLUSTER;
+            cluster = cluster || M[i0 + j] > CHECK_ROWS;
             g.M[j] = M[i0 + j];
             g.alpha[j] = alpha[i0 + j];
             g.chi_hat[j] = chi_hat[i0 + j];
@@ -249,8 +251,10 @@ cudaError_t launch_check_compact_grouped(int n, int words, const int64_t* M, con
             g.cs[j] = cs[i0 + j];
         }
         const cudaError_t e =
-            launch_dependent_cluster(words == 1 ? check_compact_group_kernel<1> : check_compact_group_kernel<2>,
-                                     dim3(g.count * blocks), dim3(NT), blocks, st, g);
+            cluster ? launch_dependent_cluster(words == 1 ? check_compact_group_kernel<1, true> : check_compact_group_kernel<2, true>,
+                                               dim3(g.count * CHECK_CLUSTER), dim3(NT), CHECK_CLUSTER, st, g)
+                    : launch_dependent(words == 1 ? check_compact_group_kernel<1, false> : check_compact_group_kernel<2, false>,
+                                       dim3(g.count), dim3(NT), 0, st, g);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

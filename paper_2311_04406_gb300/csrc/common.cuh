@@ -32,7 +32,6 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster,
                                             cudaStream_t st, Args... args) {
-    if (cluster == 1) return launch_dependent(kernel, grid, block, 0, st, args...);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
