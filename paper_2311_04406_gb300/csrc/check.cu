@@ -62,14 +62,14 @@ __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const
         T x[U], d[U], m[U];
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            x[i] = ldg_elem<W>(chi_hat, r + i * step);
-            d[i] = ldg_elem<W>(Dc, r + i * step);
-            m[i] = ldg_elem<W>(mDc, r + i * step);
+            x[i] = ld_elem<W>(chi_hat, r + i * step);
+            d[i] = ld_elem<W>(Dc, r + i * step);
+            m[i] = ld_elem<W>(mDc, r + i * step);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) acc += x[i] * (a * d[i] - m[i]);
     }
-    for (; r < M; r += step) acc += ldg_elem<W>(chi_hat, r) * (a * ldg_elem<W>(Dc, r) - ldg_elem<W>(mDc, r));
+    for (; r < M; r += step) acc += ld_elem<W>(chi_hat, r) * (a * ld_elem<W>(Dc, r) - ld_elem<W>(mDc, r));
     T tot = block_sum<W>(acc);
     if constexpr (CLUSTER) {
         __shared__ T part;
@@ -131,13 +131,13 @@ __device__ __forceinline__ void sweep(int64_t n, const u64* Wm, const u64* mW, F
         T w[U], m[U];
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-            w[j] = ldg_elem<W>(Wm, i + j * step);
-            m[j] = ldg_elem<W>(mW, i + j * step);
+            w[j] = ld_elem<W>(Wm, i + j * step);
+            m[j] = ld_elem<W>(mW, i + j * step);
         }
 #pragma unroll
         for (int j = 0; j < U; ++j) f(i + j * step, w[j], m[j]);
     }
-    for (; i < n; i += step) f(i, ldg_elem<W>(Wm, i), ldg_elem<W>(mW, i));
+    for (; i < n; i += step) f(i, ld_elem<W>(Wm, i), ld_elem<W>(mW, i));
 }
 
 template <int W>
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(NT) batchrec_partial_kernel(int64_t n, const u
     const T a = ld_elem<W>(alpha, 0);
     T acc = 0;
     sweep<W>(n, Wm, mW, [&](int64_t i, T w, T m) {
-        const T x = ldg_elem<W>(chi, i);
+        const T x = ld_elem<W>(chi, i);
         acc += m * x - a * (w * x);
     });
     T tot = block_sum<W>(acc);
@@ -196,10 +196,10 @@ __global__ void __launch_bounds__(NT) batchrec_mask_kernel(int64_t n, const u64*
     ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
-        T v = ldg_elem<W>(X, i) + ldg_elem<W>(R, i);
-        T t = ldg_elem<W>(mX, i) + ldg_elem<W>(mR, i);
-        if (A) v -= ldg_elem<W>(A, i);
-        if (mA) t -= ldg_elem<W>(mA, i);
+        T v = ld_elem<W>(X, i) + ld_elem<W>(R, i);
+        T t = ld_elem<W>(mX, i) + ld_elem<W>(mR, i);
+        if (A) v -= ld_elem<W>(A, i);
+        if (mA) t -= ld_elem<W>(mA, i);
         st_elem<W>(Wo, i, v);
         st_elem<W>(mWo, i, t);
     }

@@ -55,22 +55,17 @@ template <int W> struct Elem;
 template <> struct Elem<1> { using T = u64; };
 template <> struct Elem<2> { using T = u128; };
 
+// An ordinary load.  Nearly every kernel here is launched as a dependent and may
+// be resident while the kernels before it still write its operands, so no load is
+// made through the non-coherent path (ld.global.nc, __ldg), which is for data that
+// nothing writes in the kernel's lifetime and which the compiler may move above
+// grid_dep_wait().
 template <int W>
 __device__ __forceinline__ typename Elem<W>::T ld_elem(const u64* p, int64_t i) {
     if constexpr (W == 1) {
         return p[i];
     } else {
         ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + 2 * i);
-        return (u128)v.x | ((u128)v.y << 64);
-    }
-}
-
-template <int W>
-__device__ __forceinline__ typename Elem<W>::T ldg_elem(const u64* p, int64_t i) {
-    if constexpr (W == 1) {
-        return __ldg(p + i);
-    } else {
-        ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p + 2 * i));
         return (u128)v.x | ((u128)v.y << 64);
     }
 }
@@ -87,6 +82,13 @@ __device__ __forceinline__ void st_elem(u64* p, int64_t i, typename Elem<W>::T v
     }
 }
 
+// 16-byte load at this point of the program (a plain one is moved about by the
+// compiler: the CompactTag rows kernel then took 76 registers in place of 62)
+__device__ __forceinline__ ulonglong2 ld_pair(const u64* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
 // streaming (evict-first) 16-byte load / store for data read or written once
 __device__ __forceinline__ ulonglong2 ld_stream2(const u64* p) {
     ulonglong2 v;

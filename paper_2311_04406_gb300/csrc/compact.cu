@@ -159,7 +159,7 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
         const int64_t base = row * p.N;
         if constexpr (VEC == 2) {
             for (int64_t c = c0 + 2 * lane; c < c1; c += 64) {
-                ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(p.chi + c));
+                ulonglong2 x = ld_pair(p.chi + c);
                 ulonglong2 r = ld_stream2(p.mR + base + c);
                 ulonglong2 d = ld_stream2(p.Dt + base + c);
                 ulonglong2 m = ld_stream2(p.mC + base + c);
@@ -175,10 +175,10 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
             }
         } else {
             for (int64_t c = c0 + lane; c < c1; c += 32) {
-                T x = ldg_elem<W>(p.chi, c);
-                T r = ldg_elem<W>(p.mR, base + c);
-                T d = ldg_elem<W>(p.Dt, base + c);
-                T m = ldg_elem<W>(p.mC, base + c);
+                T x = ld_elem<W>(p.chi, c);
+                T r = ld_elem<W>(p.mR, base + c);
+                T d = ld_elem<W>(p.Dt, base + c);
+                T m = ld_elem<W>(p.mC, base + c);
                 s1 += r * x;
                 s2 += d * x;
                 s3 += m * x;
@@ -197,7 +197,7 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
         const int64_t base = row * p.N;
         if constexpr (VEC == 2) {
             for (int64_t c = c0 + 2 * lane; c < c1; c += 64) {
-                ulonglong2 x = __ldg(reinterpret_cast<const ulonglong2*>(p.chi + c));
+                ulonglong2 x = ld_pair(p.chi + c);
                 ulonglong2 b = ld_stream2(p.mB + base + c);
                 ulonglong2 f = ld_stream2(p.F + base + c);
                 s1 += b.x * x.x + b.y * x.y;
@@ -205,9 +205,9 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
             }
         } else {
             for (int64_t c = c0 + lane; c < c1; c += 32) {
-                T x = ldg_elem<W>(p.chi, c);
-                s1 += ldg_elem<W>(p.mB, base + c) * x;
-                s2 += ldg_elem<W>(p.F, base + c) * x;
+                T x = ld_elem<W>(p.chi, c);
+                s1 += ld_elem<W>(p.mB, base + c) * x;
+                s2 += ld_elem<W>(p.F, base + c) * x;
             }
         }
         s1 = warp_sum<W>(s1);
@@ -302,8 +302,8 @@ __device__ __forceinline__ void vec_body(const VecParams& p, int wpr, int64_t bl
         if constexpr (VEC == 2) {
 #pragma unroll 4
             for (int64_t k = 2 * (sub * 32 + lane); k < p.K; k += 64 * wpr) {
-                ulonglong2 e = __ldg(reinterpret_cast<const ulonglong2*>(p.E + base + k));
-                ulonglong2 ma = __ldg(reinterpret_cast<const ulonglong2*>(p.mA + base + k));
+                ulonglong2 e = *reinterpret_cast<const ulonglong2*>(p.E + base + k);
+                ulonglong2 ma = *reinterpret_cast<const ulonglong2*>(p.mA + base + k);
                 ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p.vmb + k);
                 ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p.vf + k);
                 acc += e.x * w.x + e.y * w.y;
@@ -319,8 +319,8 @@ __device__ __forceinline__ void vec_body(const VecParams& p, int wpr, int64_t bl
                 for (int i = 0; i < 4; ++i) {
                     const int64_t j = k + i * step;
                     const bool in = j < p.K;
-                    e[i] = in ? ldg_elem<W>(p.E, base + j) : (T)0;
-                    a[i] = in ? ldg_elem<W>(p.mA, base + j) : (T)0;
+                    e[i] = in ? ld_elem<W>(p.E, base + j) : (T)0;
+                    a[i] = in ? ld_elem<W>(p.mA, base + j) : (T)0;
                     w[i] = in ? ld_elem<W>(p.vmb, j) : (T)0;
                     u[i] = in ? ld_elem<W>(p.vf, j) : (T)0;
                 }
@@ -373,8 +373,8 @@ __device__ __forceinline__ void vec4_body(const VecParams& p, int64_t blk) {
             T e[4], a[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                e[i] = ldg_elem<W>(p.E, base[i] + k);
-                a[i] = ldg_elem<W>(p.mA, base[i] + k);
+                e[i] = ld_elem<W>(p.E, base[i] + k);
+                a[i] = ld_elem<W>(p.mA, base[i] + k);
             }
             const T w = ld_elem<W>(p.vmb, k), u = ld_elem<W>(p.vf, k);
 #pragma unroll
@@ -404,8 +404,8 @@ __device__ __forceinline__ void vec_small_body(const VecParams& p, int64_t blk) 
 #pragma unroll 4
         for (int64_t k = l; k < p.K; k += 8) {
             const T u = ld_elem<W>(p.vf, k);
-            acc[i] += ldg_elem<W>(p.E, r * p.K + k) * vec_w<W, FORM>(ld_elem<W>(p.vmb, k), u, alpha) +
-                      ldg_elem<W>(p.mA, r * p.K + k) * u;
+            acc[i] += ld_elem<W>(p.E, r * p.K + k) * vec_w<W, FORM>(ld_elem<W>(p.vmb, k), u, alpha) +
+                      ld_elem<W>(p.mA, r * p.K + k) * u;
         }
     }
 #pragma unroll

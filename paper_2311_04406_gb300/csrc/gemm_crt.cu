@@ -768,6 +768,14 @@ __device__ __forceinline__ uint32_t reduce2(uint32_t v, uint32_t ip, uint32_t np
     return q;
 }
 
+// 16-byte load at this point of the program (plain ones are moved about by the
+// compiler: the split sums below then spilled 100 bytes)
+__device__ __forceinline__ uint4 ld_vec(const uint8_t* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 template <typename T>
 __device__ __forceinline__ T shfl_xor_elem(T v, int o) {
     if constexpr (sizeof(T) == 8) {
@@ -833,9 +841,9 @@ __global__ void __launch_bounds__(256, W == 1 ? 4 : 3) combine_kernel(const __gr
             uint4 v = make_uint4(0, 0, 0, 0);
             if (m < NP) {
                 const uint8_t* a = src + (int64_t)m * p.splits * stride;
-                v = __ldg(reinterpret_cast<const uint4*>(a));
+                v = ld_vec(a);
                 for (int s = 1; s < p.splits; ++s) {
-                    const uint4 y = __ldg(reinterpret_cast<const uint4*>(a + s * stride));
+                    const uint4 y = ld_vec(a + s * stride);
                     v = make_uint4(add2(v.x, y.x), add2(v.y, y.y), add2(v.z, y.z), add2(v.w, y.w));
                 }
                 const uint32_t ip = tab<W>().ip2[m], np = tab<W>().np2[m];
@@ -877,22 +885,21 @@ __global__ void __launch_bounds__(256, W == 1 ? 4 : 3) combine_kernel(const __gr
                 for (int n = 0; n < W; ++n) {
                     const int d0 = __float2int_rn(__fmaf_rn(qf, P[n][0], d[n][2 * v]));
                     const int d1 = __float2int_rn(__fmaf_rn(qf, P[n][1], d[n][2 * v + 1]));
-                    const long long e = (long long)d0 + (long long)d1 * 2048;
-                    if (8 * n + 2 * t < OUT) s += (T)e << (88 * n + 22 * t);
+                    const long long w = (long long)d0 + (long long)d1 * 2048;
+                    if (8 * n + 2 * t < OUT) s += (T)w << (88 * n + 22 * t);
                 }
                 part[2 * h + v] = s;
             }
         }
+        // this lane's output; its addend arrives during the exchange below
+        const int64_t ar = a0 + r + t, bc = b0 + g, e = p.swap ? bc * p.N + ar : ar * p.N + bc;
+        const T c = p.C && ar < na && bc < nb ? ld_elem<W>(p.C, e) : (T)0;
         // lane t keeps row r + t: pairs exchange halves, then the pairs' halves
         const bool t0 = t & 1, t1 = t & 2;
         const T k0 = (t0 ? part[1] : part[0]) + shfl_xor_elem<T>(t0 ? part[0] : part[1], 1);
         const T k1 = (t0 ? part[3] : part[2]) + shfl_xor_elem<T>(t0 ? part[2] : part[3], 1);
         const T z = (t1 ? k1 : k0) + shfl_xor_elem<T>(t1 ? k0 : k1, 2);
-        const int64_t ar = a0 + r + t, bc = b0 + g;
-        if (ar < na && bc < nb) {
-            const int64_t e = p.swap ? bc * p.N + ar : ar * p.N + bc;
-            st_elem<W>(p.Z, e, z + (p.C ? ldg_elem<W>(p.C, e) : (T)0));
-        }
+        if (ar < na && bc < nb) st_elem<W>(p.Z, e, z + c);
     }
 }
 

@@ -57,10 +57,10 @@ __device__ __forceinline__ typename Elem<W>::T left(const GemmArgs& a, typename 
                                                    int64_t m, int64_t kv) {
     using T = typename Elem<W>::T;
     if (a.one_half) kv += a.K;
-    if (kv < a.K) return ldg_elem<W>(a.E, m * a.K + kv);
+    if (kv < a.K) return ld_elem<W>(a.E, m * a.K + kv);
     const int64_t kx = kv - a.K;
-    T v = ldg_elem<W>(a.X, m * a.K + kx);
-    if (a.coef != COEF_ZERO) v += c * ldg_elem<W>(a.E, m * a.K + kx);
+    T v = ld_elem<W>(a.X, m * a.K + kx);
+    if (a.coef != COEF_ZERO) v += c * ld_elem<W>(a.E, m * a.K + kx);
     return v;
 }
 
@@ -100,12 +100,20 @@ __device__ __forceinline__ void cluster_sums(const typename Elem<W>::T* part, in
     ptx::cluster_sync();        // and read, before a block leaves
 }
 
-// Z = C + sum, or Z += sum where several clusters share the output
+// element e of the addend; 0 where Z += sum (Z was set to C) or there is none.
+// A thread reads the addend of all of its outputs before it stores the first, so
+// that the loads are in flight together.
+template <int W>
+__device__ __forceinline__ typename Elem<W>::T addend(const GemmArgs& a, int64_t e, int atomic) {
+    using T = typename Elem<W>::T;
+    return a.C && !atomic ? ld_elem<W>(a.C, e) : (T)0;
+}
+
+// Z = sum (the addend included), or Z += sum where several blocks share the output
 template <int W>
 __device__ __forceinline__ void put(const GemmArgs& a, int64_t e, typename Elem<W>::T v, int atomic) {
-    using T = typename Elem<W>::T;
     if (atomic) atomic_add_elem<W>(a.Z, e, v);
-    else st_elem<W>(a.Z, e, (a.C ? ldg_elem<W>(a.C, e) : (T)0) + v);
+    else st_elem<W>(a.Z, e, v);
 }
 
 // The operands of the next K slice are loaded while the present one is
@@ -146,7 +154,7 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
         const int64_t n = n0 + idx % BN, kv = k0 + idx / BN;
         if (n >= N || kv >= kend) return (T)0;
         const int64_t kq = kv + kr;
-        return kq < K ? ldg_elem<W>(a.B, kq * N + n) : ldg_elem<W>(a.F, (kq - K) * N + n);
+        return kq < K ? ld_elem<W>(a.B, kq * N + n) : ld_elem<W>(a.F, (kq - K) * N + n);
     };
     auto multiply = [&] {
 #pragma unroll 4
@@ -199,19 +207,22 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
         for (int j = 0; j < 4; ++j) Rs[ty][tx + 16 * j] = acc[0][j];
         cluster_sums<W>(&Rs[0][0], BM_SMALL * BN, [&](int i, T v) {
             const int64_t m = m0 + i / BN, n = n0 + i % BN;
-            if (m < M && n < N) put<W>(a, m * N + n, v, 0);
+            if (m < M && n < N) put<W>(a, m * N + n, v + addend<W>(a, m * N + n, 0), 0);
         });
     } else {
+        auto each = [&](auto f) {
 #pragma unroll
-        for (int i = 0; i < RI; ++i) {
-            int64_t m = m0 + ty + 16 * i;
-            if (m >= M) continue;
+            for (int i = 0; i < RI; ++i) {
+                const int64_t m = m0 + ty + 16 * i;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int64_t n = n0 + tx + 16 * j;
-                if (n < N) put<W>(a, m * N + n, acc[i][j], atomic);
+                for (int j = 0; j < 4; ++j) {
+                    const int64_t n = n0 + tx + 16 * j;
+                    if (m < M && n < N) f(acc[i][j], m * N + n);
+                }
             }
-        }
+        };
+        each([&](T& v, int64_t e) { v += addend<W>(a, e, atomic); });
+        each([&](T& v, int64_t e) { put<W>(a, e, v, atomic); });
     }
 }
 
@@ -251,11 +262,11 @@ __global__ void __launch_bounds__(NT) ring_gemv_wide_kernel(GemmArgs a, int64_t 
                 const u64* row = kv < K ? a.B + kv * N * W : a.F + (kv - K) * N * W;
                 T r[VEC];
                 if constexpr (VEC == 2) {
-                    const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(row + n));
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + n);
                     r[0] = v.x;
                     r[1] = v.y;
                 } else {
-                    r[0] = ldg_elem<W>(row, n);
+                    r[0] = ld_elem<W>(row, n);
                 }
 #pragma unroll
                 for (int i = 0; i < MM; ++i)
@@ -265,11 +276,15 @@ __global__ void __launch_bounds__(NT) ring_gemv_wide_kernel(GemmArgs a, int64_t 
         }
         __syncthreads();
     }
+    auto each = [&](auto f) {
 #pragma unroll
-    for (int v = 0; v < VEC; ++v)
+        for (int v = 0; v < VEC; ++v)
 #pragma unroll
-        for (int i = 0; i < MM; ++i)
-            if (i < M && n + v < N) put<W>(a, (int64_t)i * N + n + v, acc[i][v], atomic);
+            for (int i = 0; i < MM; ++i)
+                if (i < M && n + v < N) f(acc[i][v], (int64_t)i * N + n + v);
+    };
+    each([&](T& v, int64_t e) { v += addend<W>(a, e, atomic); });
+    each([&](T& v, int64_t e) { put<W>(a, e, v, atomic); });
 }
 
 // GEMV (M <= GV_M): a block covers 32 lanes x VEC output columns (VEC = 2: two
@@ -314,11 +329,11 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
                 const u64* row = kv < K ? a.B + kv * N * W : a.F + (kv - K) * N * W;
                 T r[VEC];
                 if constexpr (VEC == 2) {
-                    const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(row + n));
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + n);
                     r[0] = v.x;
                     r[1] = v.y;
                 } else {
-                    r[0] = ldg_elem<W>(row, n);
+                    r[0] = ld_elem<W>(row, n);
                 }
 #pragma unroll
                 for (int i = 0; i < MM; ++i)
@@ -344,11 +359,15 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
 #pragma unroll
                 for (int v = 0; v < VEC; ++v) acc[i][v] += red[w][i][lane * VEC + v];
         if (ptx::cluster_size() == 1) {
+            auto each = [&](auto f) {
 #pragma unroll
-            for (int i = 0; i < MM; ++i)
+                for (int i = 0; i < MM; ++i)
 #pragma unroll
-                for (int v = 0; v < VEC; ++v)
-                    if (i < M && n + v < N) put<W>(a, (int64_t)i * N + n + v, acc[i][v], atomic);
+                    for (int v = 0; v < VEC; ++v)
+                        if (i < M && n + v < N) f(acc[i][v], (int64_t)i * N + n + v);
+            };
+            each([&](T& v, int64_t e) { v += addend<W>(a, e, atomic); });
+            each([&](T& v, int64_t e) { put<W>(a, e, v, atomic); });
         } else {
 #pragma unroll
             for (int i = 0; i < MM; ++i)
@@ -360,7 +379,7 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
     cluster_sums<W>(part, MM * NCOL, [&](int i, T v) {
         const int row = i / NCOL;
         const int64_t col = (int64_t)blockIdx.x * NCOL + i % NCOL;
-        if (row < M && col < N) put<W>(a, row * N + col, v, atomic);
+        if (row < M && col < N) put<W>(a, row * N + col, v + addend<W>(a, row * N + col, 0), 0);
     });
 }
 

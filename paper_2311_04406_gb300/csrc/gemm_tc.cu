@@ -379,6 +379,32 @@ template <int G> struct PrologueGroup {
     int grid;                 // CTAs of the GEMM launch
 };
 
+// Z = C (0 without an addend) on the TR x TC tile at (m0, n0), by 256 threads in
+// 16-byte vectors: two elements of one row for W = 1 (N is even), one element
+// for W = 2; the loads of two vectors are in flight together.
+template <int W, int TR, int TC>
+__device__ __forceinline__ void preset_tile(const u64* C, u64* Z, int64_t M, int64_t N, int64_t m0, int64_t n0,
+                                            int tid) {
+    constexpr int VPR = TC * W / 2, U = 2;       // vectors per tile row
+    static_assert(TR * VPR % (256 * U) == 0, "whole batches");
+    const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(C);
+    ulonglong2* z2 = reinterpret_cast<ulonglong2*>(Z);
+    for (int q0 = tid; q0 < TR * VPR; q0 += 256 * U) {
+        ulonglong2 v[U];
+        int64_t at[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int q = q0 + 256 * i, r = q / VPR, j = q - r * VPR;
+            const int64_t m = m0 + r, n = n0 + (int64_t)j * 2 / W;
+            at[i] = m < M && n < N ? (m * N + n) * W / 2 : -1;
+            v[i] = C && at[i] >= 0 ? c2[at[i]] : make_ulonglong2(0, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+            if (at[i] >= 0) z2[at[i]] = v[i];
+    }
+}
+
 // thread `id` of `nthreads` working for one layer: digit planes of L in
 // R-row tiles; output tiles of R x ND (or, WIDE, ND x WIDE_COLS) for the Z = C
 // preset
@@ -391,18 +417,12 @@ __device__ __forceinline__ void prologue_body(const PrologueParams& p, int grid,
     {
         // Z = C (0 without an addend) on split tiles: their pieces are added
         // atomically.  A tile one CTA computes whole is written by that CTA.
-        // 16-byte vectors: two elements of one row for W = 1 (N is even),
-        // one element for W = 2.
-        // Blocks take tiles in turn; a split tile's TR x TC block is copied by
-        // the 256 threads, TC W / 2 vectors per row.  (A wide tile's first
-        // index counts column tiles, its second row tiles.)
+        // Blocks take tiles in turn.  (A wide tile's first index counts column
+        // tiles, its second row tiles.)
         constexpr int ND = Cfg<W>::ND;
         constexpr int TR = WIDE ? ND : R, TC = WIDE ? WIDE_COLS : ND;
-        constexpr int VPR = TC * W / 2;                      // 16-byte vectors per tile row
         const int64_t blk = id >> 8, nblk = nthreads >> 8;
         const int tid = (int)(id & 255);
-        const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(p.C);
-        ulonglong2* z2 = reinterpret_cast<ulonglong2*>(p.Z);
         const int64_t T = p.m_tiles * p.n_tiles;
         const Sched sc = sched_of(T * p.I, p.I, grid);
         for (int64_t t = blk; t < T; t += nblk) {
@@ -411,14 +431,7 @@ __device__ __forceinline__ void prologue_body(const PrologueParams& p, int grid,
             int64_t ta, tb;
             tile_mn(t, p.m_tiles, p.n_tiles, p.gm, &ta, &tb);
             const int64_t mt = WIDE ? tb : ta, nt = WIDE ? ta : tb;
-            for (int q = tid; q < TR * VPR; q += 256) {
-                const int r = q / VPR, j = q - r * VPR;
-                const int64_t m = mt * TR + r;
-                const int64_t n = nt * TC + (int64_t)j * 2 / W;
-                if (m >= p.M || n >= p.N) continue;
-                const int64_t i = (m * p.N + n) * W / 2;     // vector index
-                z2[i] = c2 ? __ldg(c2 + i) : make_ulonglong2(0, 0);
-            }
+            preset_tile<W, TR, TC>(p.C, p.Z, p.M, p.N, mt * TR, nt * TC, tid);
         }
     }
     // 2 R threads per (tile, stage): thread = (8-row group rg, K half kg, row r)
@@ -443,7 +456,7 @@ __device__ __forceinline__ void prologue_body(const PrologueParams& p, int grid,
             const ulonglong2* src = reinterpret_cast<const ulonglong2*>(base);
 #pragma unroll
             for (int e = 0; e < 4 * W; ++e) {
-                ulonglong2 v = __ldg(src + e);
+                const ulonglong2 v = src[e];
                 x[2 * e] = v.x;
                 x[2 * e + 1] = v.y;
             }
@@ -452,7 +465,7 @@ __device__ __forceinline__ void prologue_body(const PrologueParams& p, int grid,
             for (int e = 0; e < 8; ++e)
                 if (kk + e < p.K) {
 #pragma unroll
-                    for (int h = 0; h < W; ++h) x[W * e + h] = __ldg(base + W * e + h);
+                    for (int h = 0; h < W; ++h) x[W * e + h] = base[W * e + h];
                 }
         }
         if (!first_half && p.coef != COEF_ZERO) {
@@ -460,13 +473,13 @@ __device__ __forceinline__ void prologue_body(const PrologueParams& p, int grid,
                 const u64 c = p.coef == COEF_ONE ? 1ull : p.alpha[0];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
-                    if (kk + e < p.K) x[e] += c * __ldg(ebase + e);
+                    if (kk + e < p.K) x[e] += c * ebase[e];
             } else {
                 const u128 c = p.coef == COEF_ONE ? (u128)1 : ((u128)p.alpha[0] | ((u128)p.alpha[1] << 64));
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     if (kk + e >= p.K) continue;
-                    const u128 ev = (u128)__ldg(ebase + 2 * e) | ((u128)__ldg(ebase + 2 * e + 1) << 64);
+                    const u128 ev = (u128)ebase[2 * e] | ((u128)ebase[2 * e + 1] << 64);
                     const u128 xv = ((u128)x[2 * e] | ((u128)x[2 * e + 1] << 64)) + c * ev;
                     x[2 * e] = (u64)xv;
                     x[2 * e + 1] = (u64)(xv >> 64);
@@ -1497,7 +1510,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_wide_kernel(const __
 #pragma unroll
                     for (int i = 0; i < BATCH; ++i) {
                         const int64_t m = mb + c0 + i;
-                        cv[i] = (whole && p.C && m < p.M && n < p.N) ? ldg_elem<W>(p.C, m * p.N + n) : (Sum)0;
+                        cv[i] = (whole && p.C && m < p.M && n < p.N) ? ld_elem<W>(p.C, m * p.N + n) : (Sum)0;
                     }
 #pragma unroll
                     for (int i = 0; i < BATCH; ++i) {
@@ -1589,11 +1602,8 @@ __device__ __forceinline__ void prologue_r_body(const PrologueRParams& p, int gr
     constexpr int NDIG = Cfg<W>::NDIG, ND = Cfg<W>::ND;
     {
         // Z = C on split tiles (as the row-tile prologue does)
-        constexpr int VPR = ND * W / 2;
         const int64_t blk = id >> 8, nblk = nthreads >> 8;
         const int tid = (int)(id & 255);
-        const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(p.C);
-        ulonglong2* z2 = reinterpret_cast<ulonglong2*>(p.Z);
         const int64_t T = p.m_tiles * p.n_tiles;
         const Sched sc = sched_of(T * p.I, p.I, grid);
         for (int64_t t = blk; t < T; t += nblk) {
@@ -1601,14 +1611,7 @@ __device__ __forceinline__ void prologue_r_body(const PrologueRParams& p, int gr
             if (u + p.I <= range_end_of(sc, u)) continue;
             int64_t mt, nt;
             tile_mn(t, p.m_tiles, p.n_tiles, p.gm, &mt, &nt);
-            for (int q = tid; q < BM * VPR; q += 256) {
-                const int r = q / VPR, j = q - r * VPR;
-                const int64_t m = mt * BM + r;
-                const int64_t n = nt * ND + (int64_t)j * 2 / W;
-                if (m >= p.M || n >= p.N) continue;
-                const int64_t i = (m * p.N + n) * W / 2;
-                z2[i] = c2 ? __ldg(c2 + i) : make_ulonglong2(0, 0);
-            }
+            preset_tile<W, BM, ND>(p.C, p.Z, p.M, p.N, mt * BM, nt * ND, tid);
         }
     }
     const int64_t per_tile = (int64_t)p.S_tot * 2 * ND;
@@ -1629,8 +1632,8 @@ __device__ __forceinline__ void prologue_r_body(const PrologueRParams& p, int gr
         T v = 0;
         if (n < p.N && kk + e < p.K) {
             const int64_t i = (kk + e) * p.N + n;
-            v = ldg_elem<W>(first ? p.B : p.F, i);
-            if (first && p.coef != COEF_ZERO) v += cv * ldg_elem<W>(p.F, i);
+            v = ld_elem<W>(first ? p.B : p.F, i);
+            if (first && p.coef != COEF_ZERO) v += cv * ld_elem<W>(p.F, i);
         }
         x[W * e] = (u64)v;
         if constexpr (W == 2) x[W * e + 1] = (u64)(v >> 64);
@@ -1937,28 +1940,39 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_tall_kernel(const __
                         // the row's ND sums as 16-byte vectors (N is even for W = 1)
                         ulonglong2* z2 = reinterpret_cast<ulonglong2*>(p.Z + e0 * W);
                         const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(p.C + e0 * W);
-                        constexpr int V = ND * W / 2;
+                        constexpr int V = ND * W / 2, BATCH = 4;   // loads of the addend in flight together
 #pragma unroll
-                        for (int q = 0; q < V; ++q) {
-                            const ulonglong2 cq = p.C ? __ldg(c2 + q) : make_ulonglong2(0, 0);
-                            ulonglong2 o;
-                            if constexpr (W == 1) {
-                                o.x = cq.x + sum[2 * q];
-                                o.y = cq.y + sum[2 * q + 1];
-                            } else {
-                                const Sum r = ((Sum)cq.x | ((Sum)cq.y << 64)) + sum[q];
-                                o.x = (u64)r;
-                                o.y = (u64)(r >> 64);
+                        for (int q0 = 0; q0 < V; q0 += BATCH) {
+                            ulonglong2 cv[BATCH];
+#pragma unroll
+                            for (int i = 0; i < BATCH; ++i) cv[i] = p.C ? c2[q0 + i] : make_ulonglong2(0, 0);
+#pragma unroll
+                            for (int i = 0; i < BATCH; ++i) {
+                                const int q = q0 + i;
+                                ulonglong2 o;
+                                if constexpr (W == 1) {
+                                    o.x = cv[i].x + sum[2 * q];
+                                    o.y = cv[i].y + sum[2 * q + 1];
+                                } else {
+                                    const Sum r = ((Sum)cv[i].x | ((Sum)cv[i].y << 64)) + sum[q];
+                                    o.x = (u64)r;
+                                    o.y = (u64)(r >> 64);
+                                }
+                                z2[q] = o;
                             }
-                            z2[q] = o;
                         }
                     } else {
+                        if (whole && p.C) {      // loads of the addend before the first store
+#pragma unroll
+                            for (int c = 0; c < ND; ++c)
+                                if (n0 + c < p.N) sum[c] += ld_elem<W>(p.C, e0 + c);
+                        }
 #pragma unroll
                         for (int c = 0; c < ND; ++c) {
                             if (n0 + c >= p.N) break;
                             const int64_t e = e0 + c;
                             if (whole) {
-                                st_elem<W>(p.Z, e, (p.C ? ldg_elem<W>(p.C, e) : (Sum)0) + sum[c]);
+                                st_elem<W>(p.Z, e, sum[c]);
                             } else {
                                 if constexpr (W == 1) red_add_u64(p.Z + e, sum[c]);
                                 else atomic_add_u128(p.Z + 2 * e, sum[c]);

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(NT) im2col_kernel(const Im2colArgs a, uint32_t
             const uint32_t y = oy * a.stride + ky - a.pad, x = ox * a.stride + kx - a.pad;
             v[j] = 0;
             if (j * step < end - row && y < a.H && x < a.W)
-                v[j] = ldg_elem<WW>(a.in, (((int64_t)b * a.C + c) * a.H + y) * a.W + x);
+                v[j] = ld_elem<WW>(a.in, (((int64_t)b * a.C + c) * a.H + y) * a.W + x);
             for (ox += step; ox >= a.Wo; ox -= a.Wo)
                 if (++oy == a.Ho) {
                     oy = 0;

@@ -41,14 +41,14 @@ __global__ void __launch_bounds__(NT) lincomb_kernel(const __grid_constant__ Lin
                 st_stream2(a.out + 2 * i, make_ulonglong2(x, y));
             } else {
                 u64 x = 0;
-                for (int j = 0; j < a.count; ++j) x += (u64)a.coef[j] * ldg_elem<1>(a.in[j], i);
+                for (int j = 0; j < a.count; ++j) x += (u64)a.coef[j] * ld_elem<1>(a.in[j], i);
                 st_elem<1>(a.out, i, x);
             }
         }
     } else {
         for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * NT) {
             T x = 0;
-            for (int j = 0; j < a.count; ++j) x += (T)(__int128)a.coef[j] * ldg_elem<W>(a.in[j], i);
+            for (int j = 0; j < a.count; ++j) x += (T)(__int128)a.coef[j] * ld_elem<W>(a.in[j], i);
             st_elem<W>(a.out, i, x);
         }
     }
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(NT) lincomb_group_kernel(const __grid_constant
     const int64_t end = base + GROUP_ELEMS < a.n[g] ? base + GROUP_ELEMS : a.n[g];
     for (int64_t i = base + threadIdx.x; i < end; i += NT) {
         T x = 0;
-        for (int j = 0; j < a.count; ++j) x += (T)(__int128)a.coef[j] * ldg_elem<W>(a.in[g][j], i);
+        for (int j = 0; j < a.count; ++j) x += (T)(__int128)a.coef[j] * ld_elem<W>(a.in[g][j], i);
         st_elem<W>(a.out[g], i, x);
     }
 }

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(TILE * ROWS) transpose_kernel(int64_t rows, in
 #pragma unroll
     for (int j = 0; j < TILE; j += ROWS) {
         const int64_t r = r0 + ty + j, c = c0 + tx;
-        if (r < rows && c < cols) tile[ty + j][tx] = ldg_elem<W>(in, r * cols + c);
+        if (r < rows && c < cols) tile[ty + j][tx] = ld_elem<W>(in, r * cols + c);
     }
     __syncthreads();
 #pragma unroll

@@ -26,11 +26,10 @@ __global__ void __launch_bounds__(NT) optmac_trunc_kernel(int64_t MN, int k, int
     const T mk = k >= 64 * W ? ~(T)0 : (((T)1 << k) - 1);
     const T a = ld_elem<W>(alpha, 0);
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < MN; i += (int64_t)gridDim.x * NT) {
-        const T delta = (ldg_elem<W>(Dt, i) & mk) >> f;
-        const T rho = (ldg_elem<W>(P, i) & mk) >> f;
-        const T tau = rho - delta;
-        st_elem<W>(Zf, i, ldg_elem<W>(Rf, i) + (party0 ? tau : (T)0));
-        st_elem<W>(mZf, i, ldg_elem<W>(mRf, i) + a * tau);
+        const T d = ld_elem<W>(Dt, i), q = ld_elem<W>(P, i), r = ld_elem<W>(Rf, i), m = ld_elem<W>(mRf, i);
+        const T tau = ((q & mk) >> f) - ((d & mk) >> f);
+        st_elem<W>(Zf, i, r + (party0 ? tau : (T)0));
+        st_elem<W>(mZf, i, m + a * tau);
     }
 }
 
