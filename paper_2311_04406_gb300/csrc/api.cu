@@ -64,14 +64,16 @@ size_t gemm_ws(const mpc_layer* L, int one_half = 0) {
 }
 
 // 1 when the residue path runs the layer in this workspace, 0 when it does not
-// (no choice of it, or the built-in rule chose it and the workspace only covers
-// the other paths); negative status when the table demands it and it cannot.
+// (no choice of it, or the built-in rule chose it and the workspace, too small or
+// not 256-byte aligned, only serves the other paths, which then judge it by their
+// own needs: the integer pipes have none); negative status when the table demands
+// the path and it cannot run.
 int use_crt(const mpcl::Choice& c, const mpcl::GemmArgs& g, const void* ws, size_t ws_bytes) {
     if (!c.crt) return 0;
     const bool fits = ws && ws_bytes >= mpcl::gemm_crt_workspace(g.M, g.K, g.N, g.words, g.one_half);
-    if (!fits) return c.tuned ? MPC_E_WORKSPACE : 0;
-    if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return MPC_E_ALIGN;
-    return 1;
+    if (fits && reinterpret_cast<uintptr_t>(ws) % 256 == 0) return 1;
+    if (!c.tuned) return 0;
+    return fits ? MPC_E_ALIGN : MPC_E_WORKSPACE;
 }
 
 int run_gemm(mpcl::GemmArgs g, void* ws, size_t ws_bytes, cudaStream_t st) {
