@@ -200,7 +200,9 @@ int mpc_linear_tag_grouped(const mpc_layer *layers, int count, int mode, const m
                            void *workspace, size_t ws_bytes, void *stream);
 
 /* which: MPC_WS_SHARE, MPC_WS_TAG_FULL or MPC_WS_TAG_COMPACT.  0 on invalid
- * arguments (as mpc_workspace_size). */
+ * arguments (as mpc_workspace_size).  For shares and full tags: the larger of the
+ * digit planes of all layers together, which the call needs, and of the residue
+ * planes of the largest single layer, without which that layer takes another path. */
 size_t mpc_workspace_size_grouped(const mpc_layer *layers, int count, int which);
 
 /*
@@ -255,10 +257,11 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * tiles and of the integer pipes the residue path wherever its estimated time is
  * lower, which is for layers large in both output dimensions, from about 600 in
  * Z_2^64 and 256 in Z_2^128, provided that the call's workspace covers it -- a
- * smaller workspace that covers the other paths is accepted and gives the same
- * result).  mpc_autotune_choice reports the tile that those other paths use for
+ * smaller workspace that covers the other paths is accepted, whether the rule or
+ * an entry names the residue path, and gives the same result).  mpc_autotune_choice reports the tile that those other paths use for
  * untuned shapes.  The table is process-wide and thread-safe; workspace
- * sizes do not depend on it.
+ * sizes do not depend on it, but for the planes of an entry that names the residue
+ * path for a shape far from that rule.
  *
  * mpc_autotune: for each distinct shape of layers[count], times the
  *   candidates (128-row tiles, 64-row tiles for M <= 64, the wide tile for

@@ -55,33 +55,33 @@ int cuda_status(cudaError_t e) {
 }
 
 // Workspace of a GEMM: the tensor-core digit planes whenever that kernel can
-// run the shape, so that any launch-table choice fits the same workspace.
+// run the shape, so that any launch-table choice of those tiles fits the same
+// workspace, and the residue planes of shapes near or inside that path's rule or
+// with a table entry that names it.
 size_t gemm_ws(const mpc_layer* L, int one_half = 0) {
     size_t b = mpcl::gemm_tc_workspace(L->M, L->K, L->N, L->ring.words, one_half);
-    if (mpcl::gemm_crt_candidate(L->M, L->K, L->N, L->ring.words))
+    if (mpcl::gemm_crt_sized(L->M, L->K, L->N, L->ring.words))
         b = std::max(b, mpcl::gemm_crt_workspace(L->M, L->K, L->N, L->ring.words, one_half));
     return b;
 }
 
-// 1 when the residue path runs the layer in this workspace, 0 when it does not
-// (no choice of it, or the built-in rule chose it and the workspace, too small or
-// not 256-byte aligned, only serves the other paths, which then judge it by their
-// own needs: the integer pipes have none); negative status when the table demands
-// the path and it cannot run.
-int use_crt(const mpcl::Choice& c, const mpcl::GemmArgs& g, const void* ws, size_t ws_bytes) {
-    if (!c.crt) return 0;
-    const bool fits = ws && ws_bytes >= mpcl::gemm_crt_workspace(g.M, g.K, g.N, g.words, g.one_half);
-    if (fits && reinterpret_cast<uintptr_t>(ws) % 256 == 0) return 1;
-    if (!c.tuned) return 0;
-    return fits ? MPC_E_ALIGN : MPC_E_WORKSPACE;
+// Whether the residue path runs the layer in this workspace.  If it was chosen but
+// the workspace is too small or not 256-byte aligned, c becomes the choice among
+// the other paths, which judge the workspace by their own needs (the integer pipes
+// have none).
+bool use_crt(mpcl::Choice& c, const mpcl::GemmArgs& g, const void* ws, size_t ws_bytes) {
+    if (!c.crt) return false;
+    if (ws && reinterpret_cast<uintptr_t>(ws) % 256 == 0 &&
+        ws_bytes >= mpcl::gemm_crt_workspace(g.M, g.K, g.N, g.words, g.one_half))
+        return true;
+    if (c.tuned) c = mpcl::gemm_built_in(g.M, g.K, g.N, g.words);
+    return false;
 }
 
 int run_gemm(mpcl::GemmArgs g, void* ws, size_t ws_bytes, cudaStream_t st) {
     if (g.M == 0 || g.N == 0) return MPC_OK;
-    const mpcl::Choice c = mpcl::gemm_choice(g.M, g.K, g.N, g.words);
-    const int crt = use_crt(c, g, ws, ws_bytes);
-    if (crt < 0) return crt;
-    if (crt) return cuda_status(mpcl::launch_gemm_crt(g, ws, ws_bytes, st));
+    mpcl::Choice c = mpcl::gemm_choice(g.M, g.K, g.N, g.words);
+    if (use_crt(c, g, ws, ws_bytes)) return cuda_status(mpcl::launch_gemm_crt(g, ws, ws_bytes, st));
     if (c.path == 1) {
         if (!ws || ws_bytes < mpcl::gemm_tc_workspace(g.M, g.K, g.N, g.words, g.one_half))
             return MPC_E_WORKSPACE;
@@ -431,15 +431,6 @@ bool on_tc(const mpc_layer& L) {
     return L.M > 0 && L.N > 0 && mpcl::gemm_choice(L.M, L.K, L.N, L.ring.words).path == 1;
 }
 
-// Workspace of a grouped GEMM: one region per layer, each as large as the layer's
-// own call needs (whatever the launch table picks); without the residue path,
-// the digit planes alone.
-size_t region(const mpc_layer& L, bool with_crt) {
-    if (L.M == 0 || L.N == 0) return 0;
-    const size_t b = with_crt ? gemm_ws(&L) : mpcl::gemm_tc_workspace(L.M, L.K, L.N, L.ring.words);
-    return (b + 255) & ~size_t(255);
-}
-
 // The residue path in a group: a layer there runs by itself, where the digit
 // tiles share their launches, so the rule asks for a larger gain.  Z_2^64 layers
 // that the digit tiles can run stay with them unless the table says otherwise.
@@ -448,9 +439,25 @@ bool group_uses_crt(const mpcl::Choice& c, int64_t M, int64_t K, int64_t N, int 
     return (words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words)) && mpcl::gemm_crt_preferred(M, K, N, words, true);
 }
 
-size_t group_gemm_ws(const mpc_layer* layers, int count, bool with_crt) {
+// Workspace of a grouped GEMM (whatever the launch table picks): the digit planes
+// of every layer one after another, since the digit tiles run together; the planes
+// of each residue layer at the start, since those layers run one after another
+// behind the digit tiles on the same stream, and every kernel waits for the one
+// before it.
+size_t digit_region(int64_t M, int64_t K, int64_t N, int words) {
+    return M == 0 || N == 0 ? 0 : (mpcl::gemm_tc_workspace(M, K, N, words) + 255) & ~size_t(255);
+}
+
+size_t group_digit_ws(const mpc_layer* layers, int count) {
     size_t t = 0;
-    for (int i = 0; i < count; ++i) t += region(layers[i], with_crt);
+    for (int i = 0; i < count; ++i) t += digit_region(layers[i].M, layers[i].K, layers[i].N, layers[i].ring.words);
+    return t;
+}
+
+size_t group_gemm_ws(const mpc_layer* layers, int count) {
+    size_t t = group_digit_ws(layers, count);
+    for (int i = 0; i < count; ++i)
+        if (layers[i].M > 0 && layers[i].N > 0) t = std::max(t, gemm_ws(&layers[i]));
     return t;
 }
 
@@ -504,27 +511,22 @@ SidePool* side_pool() {
 
 int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, void* ws, size_t ws_bytes,
                    cudaStream_t st) {
-    // a workspace without the residue path's planes is accepted as long as no
-    // table entry demands that path
-    const bool with_crt = ws_bytes >= group_gemm_ws(layers, count, true);
-    const size_t need = group_gemm_ws(layers, count, with_crt);
+    // the digit planes have to fit; a layer whose residue planes do not takes
+    // another path
+    const size_t need = group_digit_ws(layers, count);
     if (need > 0) {
         if (!ws || ws_bytes < need) return MPC_E_WORKSPACE;
         if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) return MPC_E_ALIGN;
     }
     std::vector<mpcl::GemmArgs> tc, simt, crt;
-    std::vector<uint8_t*> ap, cp;
+    std::vector<uint8_t*> ap;
     uint8_t* cur = static_cast<uint8_t*>(ws);
     for (int i = 0; i < count; ++i) {
         if (g[i].M == 0 || g[i].N == 0) continue;
-        const mpcl::Choice c = mpcl::gemm_choice(g[i].M, g[i].K, g[i].N, g[i].words);
+        mpcl::Choice c = mpcl::gemm_choice(g[i].M, g[i].K, g[i].N, g[i].words);
         mpcl::GemmArgs x = g[i];
-        const size_t bytes = region(layers[i], with_crt);
-        const int use = group_uses_crt(c, x.M, x.K, x.N, x.words) ? use_crt(c, x, with_crt ? cur : nullptr, bytes) : 0;
-        if (use < 0) return use;
-        if (use) {
+        if (group_uses_crt(c, x.M, x.K, x.N, x.words) && use_crt(c, x, ws, ws_bytes)) {
             crt.push_back(x);
-            cp.push_back(cur);
         } else if (c.path == 1) {
             x.gm = c.gm;
             x.rows = c.rows;
@@ -535,12 +537,10 @@ int run_gemm_group(const mpc_layer* layers, int count, const mpcl::GemmArgs* g, 
             x.rows = c.rows;
             simt.push_back(x);
         }
-        cur += bytes;
+        cur += digit_region(x.M, x.K, x.N, x.words);
     }
     auto run_crt = [&]() -> int {
-        for (size_t j = 0; j < crt.size(); ++j)
-            CHK(cuda_status(mpcl::launch_gemm_crt(
-                crt[j], cp[j], mpcl::gemm_crt_workspace(crt[j].M, crt[j].K, crt[j].N, crt[j].words), st)));
+        for (const auto& x : crt) CHK(cuda_status(mpcl::launch_gemm_crt(x, ws, ws_bytes, st)));
         return MPC_OK;
     };
     const bool tensor = !tc.empty() || !crt.empty();
@@ -656,7 +656,7 @@ size_t mpc_workspace_size_grouped(const mpc_layer* layers, int count, int which)
     }
     switch (which) {
         case MPC_WS_SHARE:
-        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count, true);
+        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count);
         case MPC_WS_TAG_COMPACT: return group_compact_ws(layers, count);
         default: return 0;
     }

@@ -1046,10 +1046,12 @@ cudaError_t run(const GemmArgs& a, const CrtPlan& q, uint8_t* ws, cudaStream_t s
 
 }  // namespace
 
-bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half) {
+namespace {
+// the plan of a shape that the kernels can run
+bool feasible_plan(int64_t M, int64_t K, int64_t N, int words, int one_half, CrtPlan& q) {
     if ((words != 1 && words != 2) || M < 1 || N < 1 || K < 1) return false;
     if (2 * cdiv(K, KS) * KS > CRT_MAX_K2) return false;
-    const CrtPlan q = crt_plan(M, K, N, words, one_half);
+    q = crt_plan(M, K, N, words, one_half);
     // 32-bit block, unit and thread counts
     const double threads = (double)(q.a_tiles * 128.0 + q.b_tiles * (q.bn / 2.0)) * q.kb * 8;
     if (q.total / MAP_ROW >= (size_t(1) << 31)) return false;   // map coordinates
@@ -1061,7 +1063,6 @@ bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half)
 // (a constant, the left operand's digit planes, and the waves of Kd-deep units
 // over 152 SMs), or the integer pipes for the Z_2^64 layers with odd N that the
 // digit tiles do not take.
-namespace {
 double digit_us(int64_t M, int64_t K, int64_t N, int words) {
     if (!gemm_tc_feasible(M, K, N, words)) return 15.0 + 2.0 * M * K * N / (words == 1 ? 2.15e6 : 0.5e6);
     const int64_t nd = words == 1 ? 32 : 16, kd = words == 1 ? 128 : 64;
@@ -1073,22 +1074,23 @@ double digit_us(int64_t M, int64_t K, int64_t N, int words) {
 constexpr size_t MAX_WORKSPACE = size_t(12) << 30;
 // The residue path's time over the other paths'.  In a group the digit tiles'
 // launch, set-up and last wave are shared with the other layers.
-double crt_ratio(int64_t M, int64_t K, int64_t N, int words, bool grouped = false) {
-    if (M <= 8 || N <= 8 || !gemm_crt_feasible(M, K, N, words, 0)) return 1e9;
+// 1e9: not run there; `total`: its workspace.
+double crt_ratio(int64_t M, int64_t K, int64_t N, int words, bool grouped = false, size_t* total = nullptr) {
+    CrtPlan q;
+    if (M <= 8 || N <= 8 || !feasible_plan(M, K, N, words, 0, q) || q.total > MAX_WORKSPACE) return 1e9;
+    if (total) *total = q.total;
     // up to 64 rows the wide and 64-row digit tiles waste less than 256-row tiles
     if (M <= 64 && gemm_tc_feasible(M, K, N, words)) return 1e8;
-    const CrtPlan q = crt_plan(M, K, N, words, 0);
-    if (q.total > MAX_WORKSPACE) return 1e9;
     const double shared = grouped ? (words == 1 ? 12.0 : 18.0) : 0.0;
     return q.us / (digit_us(M, K, N, words) - shared);
 }
 }  // namespace
 
-// Shapes near or inside the rule, and small ones whose workspace is small (the
-// launch table may then demand the path).
+bool gemm_crt_near(int64_t M, int64_t K, int64_t N, int words) { return crt_ratio(M, K, N, words) < 1.1; }
 bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words) {
-    const double r = crt_ratio(M, K, N, words);
-    return r < 1.1 || (r < 1e9 && crt_plan(M, K, N, words, 0).total <= (size_t(32) << 20));
+    size_t total = 0;
+    const double r = crt_ratio(M, K, N, words, false, &total);
+    return r < 1.1 || (r < 1e9 && total <= (size_t(32) << 20));
 }
 bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words, bool grouped) {
     return M > 32 && N > 64 && crt_ratio(M, K, N, words, grouped) < 0.93;   // within the measured sizes
@@ -1099,8 +1101,8 @@ size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_ha
 }
 
 cudaError_t launch_gemm_crt(const GemmArgs& a, void* ws, size_t ws_bytes, cudaStream_t st) {
-    if (!gemm_crt_feasible(a.M, a.K, a.N, a.words, a.one_half)) return cudaErrorNotSupported;
-    const CrtPlan q = crt_plan(a.M, a.K, a.N, a.words, a.one_half);
+    CrtPlan q;
+    if (!feasible_plan(a.M, a.K, a.N, a.words, a.one_half, q)) return cudaErrorNotSupported;
     if (!ws || ws_bytes < q.total) return cudaErrorInvalidValue;
     return a.words == 1 ? run<1>(a, q, (uint8_t*)ws, st) : run<2>(a, q, (uint8_t*)ws, st);
 }

@@ -48,6 +48,7 @@ struct Choice {
     int crt;    // the residue path runs the layer when the workspace holds it
 };
 Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words);
+Choice gemm_built_in(int64_t M, int64_t K, int64_t N, int words);   // without the launch table
 int wide_tile_rows(int words);   // the launch-table value of the wide tensor-core tile
 // the launch-table value of the tall tensor-core tile (128-row tiles whose
 // left operand the GEMM converts itself)
@@ -78,10 +79,12 @@ void* tensor_map_encoder();       // the driver's cuTensorMapEncodeTiled, or NUL
 int tc_timeout_flag(bool* set);   // synchronous; 0 on success
 
 // ring GEMM from residue products (exact); layers large in both output
-// dimensions.  A candidate is a shape whose workspace covers this path, a
-// superset of the shapes the built-in rule runs on it.
-bool gemm_crt_feasible(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
+// dimensions.  Near: shapes close to or inside the built-in rule, whose workspace
+// covers this path.  Candidate: those, and small ones, which the launch table may
+// give to it; sized: near or given to it.
+bool gemm_crt_near(int64_t M, int64_t K, int64_t N, int words);
 bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words);
+bool gemm_crt_sized(int64_t M, int64_t K, int64_t N, int words);
 bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words, bool grouped = false);
 size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
 constexpr int CRT_LAUNCHES = 3;

@@ -79,6 +79,14 @@ int default_rows(int64_t M, int64_t K, int64_t N, int words) {
 
 }  // namespace
 
+Choice gemm_built_in(int64_t M, int64_t K, int64_t N, int words) {
+    Choice c{};
+    c.path = gemm_tc_eligible(M, K, N, words) ? 1 : 0;
+    c.rows = c.path == 1 ? default_rows(M, K, N, words) : 0;
+    c.crt = gemm_crt_preferred(M, K, N, words) ? 1 : 0;
+    return c;
+}
+
 Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words) {
     {
         std::lock_guard<std::mutex> lk(g_mu);
@@ -89,14 +97,14 @@ Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words) {
             return c;
         }
     }
-    Choice c;
-    c.path = gemm_tc_eligible(M, K, N, words) ? 1 : 0;
-    c.gm = 0;
-    c.waves = 0;
-    c.tuned = 0;
-    c.rows = c.path == 1 ? default_rows(M, K, N, words) : 0;
-    c.crt = gemm_crt_preferred(M, K, N, words) ? 1 : 0;
-    return c;
+    return gemm_built_in(M, K, N, words);
+}
+
+bool gemm_crt_sized(int64_t M, int64_t K, int64_t N, int words) {
+    if (gemm_crt_near(M, K, N, words)) return true;
+    std::lock_guard<std::mutex> lk(g_mu);
+    auto it = table().find(Key{words, M, K, N});
+    return it != table().end() && it->second.path == 1 && it->second.rows == CRT_TILE_ROWS;
 }
 
 }  // namespace mpcl

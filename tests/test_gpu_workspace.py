@@ -1,6 +1,6 @@
-"""What the layers of the residue path ask of the caller's workspace: the built-in
-rule takes the path only where the workspace serves it, and a call that ran
-without it (integer pipes: odd N in Z_2^64) still runs in any workspace."""
+"""What the layers of the residue path ask of the caller's workspace: they take the
+path only where the workspace serves it, and a call that ran without it (integer
+pipes: odd N in Z_2^64) still runs in any workspace."""
 import ctypes
 
 import numpy as np
@@ -32,10 +32,19 @@ def test_workspace_is_judged_by_the_path_that_runs(lib):
     # gets past validation (and fails at the launch: no GPU here)
     assert share(0x10010) == abi.MPC_E_CUDA
     assert share(None) == abi.MPC_E_CUDA
-    # an entry that demands the path is held to its workspace
+    # also when a table entry names the path
     abi.mpc_autotune_set(L, 1, tile_rows=256)
-    assert share(0x10010) == abi.MPC_E_ALIGN
-    assert share(None) == abi.MPC_E_WORKSPACE
+    assert share(0x10010) == abi.MPC_E_CUDA and share(None) == abi.MPC_E_CUDA
+    # the digit tiles judge the workspace as ever
+    L = abi.make_layer(64, 256, 256)
+    digits = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE)
+    abi.mpc_autotune_set(L, 1, tile_rows=256)
+    assert abi.mpc_workspace_size(L, abi.MPC_WS_SHARE) > digits      # its planes, for callers that ask now
+    need = digits
+    assert share(0x10100) == abi.MPC_E_CUDA
+    assert share(0x10010) == abi.MPC_E_ALIGN and share(None) == abi.MPC_E_WORKSPACE
+    need -= 1
+    assert share(0x10100) == abi.MPC_E_WORKSPACE
     abi.mpc_autotune_clear()
 
 
@@ -53,4 +62,54 @@ def test_unaligned_workspace_gives_the_same_result(lib):
         abi.mpc_linear_share(L, *x, Z, ws=ws)
         out.append(host(Z))
     assert np.array_equal(out[0], out[1])
+    assert abi.mpc_device_status() == 0
+
+
+def test_grouped_workspace_sizes(lib):
+    """The digit planes of all layers, or the residue planes of one: a group whose
+    layers run as digits reserves no residue planes for them."""
+    size = lambda shapes, bits: abi.mpc_workspace_size_grouped(      # noqa: E731
+        [abi.make_layer(*s, bits // 2, bits // 2) for s in shapes], abi.MPC_WS_SHARE)
+    for shape, bits in (((2048, 1024, 4096), 64), ((1129, 1692, 1468), 64), ((512, 512, 512), 128)):
+        one = size([shape], bits)
+        assert one == abi.mpc_workspace_size(abi.make_layer(*shape, bits // 2, bits // 2), abi.MPC_WS_SHARE)
+        digits = size([shape] * 12, bits) - size([shape] * 11, bits)
+        assert digits < one                      # the layer's own call may run as residues
+        for n in (1, 2, 6, 11):
+            assert size([shape] * n, bits) == max(one, n * digits)
+    assert size([ODD] * 9, 64) == size([ODD], 64)     # no digit planes: one set of residue planes
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ring,shapes", [
+    (synth.Z128, [(512, 512, 512), (100, 64, 48), (4, 300, 64), (400, 640, 512), (2048, 72, 32), (640, 512, 300)]),
+    (synth.Z64, [ODD, (300, 200, 96), (900, 400, 901), (20, 300, 33), (1100, 64, 66)])], ids=["z128", "z64"])
+def test_residue_layers_share_their_planes(lib, ring, shapes):
+    """Residue layers of a group in the same planes, which overlay the digit planes,
+    in every workspace from the smallest on: all on the path, some, none."""
+    import torch
+    Ls = [abi.make_layer(*s, ring.k, ring.s, 1, 2) for s in shapes]
+    data, want = [], []
+    for L, (M, K, N) in zip(Ls, shapes):
+        u = lambda tid, *s: dev(synth.uniform(M + N, tid, 0, s, ring.bits))     # noqa: E731
+        x = dict(E=u(1, M, K), F=u(2, K, N), A_i=u(3, M, K), B_i=u(4, K, N), C_i=u(5, M, N))
+        data.append(x)
+        w = empty_like_ring((M, N), ring.words)
+        abi.mpc_linear_share(L, *x.values(), w)
+        want.append(host(w))
+    full = abi.mpc_workspace_size_grouped(Ls, abi.MPC_WS_SHARE)
+    # digit planes: what a group of many copies grows by
+    many = lambda n: abi.mpc_workspace_size_grouped(Ls * n, abi.MPC_WS_SHARE)      # noqa: E731
+    digits = many(40) - many(39)
+    crt = sorted(abi.mpc_workspace_size(L, abi.MPC_WS_SHARE) for L, s in zip(Ls, shapes)
+                 if abi.mpc_launch_count(L, abi.MPC_WS_SHARE) == 3)
+    sizes = {full, max(digits, 256)} | {b for b in crt if b >= digits}
+    assert len(crt) >= 2 and len(sizes) >= 2
+    for nbytes in sorted(sizes):
+        Zs = [empty_like_ring(s[::2], ring.words) for s in shapes]
+        for rep in range(2):
+            abi.mpc_linear_share_grouped(Ls, [dict(x, Z_i=Z) for x, Z in zip(data, Zs)],
+                                         ws=torch.empty(nbytes, dtype=torch.uint8, device="cuda"))
+        for Z, w, s in zip(Zs, want, shapes):
+            assert np.array_equal(host(Z), w), (nbytes, s)
     assert abi.mpc_device_status() == 0
