@@ -281,14 +281,17 @@ class Server:
         base = req.region[0]
         return {k: self.arena.view(base + off, shape, n) for k, (shape, off, n) in req.plan[li].items()}
 
+    def _group_ws(self, layers) -> int:
+        """Workspace of a tick part's grouped calls."""
+        which = (abi.MPC_WS_SHARE, abi.MPC_WS_TAG_COMPACT if self.tag == "compact" else abi.MPC_WS_TAG_FULL)
+        return (max(abi.mpc_workspace_size_grouped(layers, w) for w in which) + 255) // 256 * 256
+
     def _layer_ws(self, M, K, N) -> int:
         key = (M, K, N, self.tag)
         need = self._ws_cache.get(key)
         if need is None:
             L = abi.make_layer(M, K, N, self.ring.k, self.ring.s, self.party, self.nparties)
-            which = (abi.MPC_WS_SHARE, abi.MPC_WS_TAG_COMPACT if self.tag == "compact" else abi.MPC_WS_TAG_FULL)
-            need = self._ws_cache[key] = (max(abi.mpc_workspace_size_grouped([L], w) for w in which)
-                                          + 255) // 256 * 256
+            need = self._ws_cache[key] = self._group_ws([L])
         return need
 
     def _parts(self, group):
@@ -296,12 +299,16 @@ class Server:
         last part may need a workspace of its own (returned size > 0)."""
         parts, part, used = [], [], 0
         for r in group:
-            need = self._layer_args(r, r.nxt)["ws_need"]
-            if part and used + need > self.ws.numel():
-                parts.append(part)
-                part, used = [], 0
+            # a part needs at most what its layers need one by one, often less
+            # (layers that run in turn share their scratch): asked for only
+            # where that sum does not fit
+            used += self._layer_args(r, r.nxt)["ws_need"]
+            if part and used > self.ws.numel():
+                used = self._group_ws([self._layer_args(q, q.nxt)["layer"] for q in part + [r]])
+                if used > self.ws.numel():
+                    parts.append(part)
+                    part, used = [], self._layer_args(r, r.nxt)["ws_need"]
             part.append(r)
-            used += need
         extra = used if (part and used > self.ws.numel()) else 0
         if part:
             parts.append(part)

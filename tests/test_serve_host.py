@@ -76,3 +76,29 @@ def test_request_stream_is_seeded_and_poisson():
     assert min(r.batch for r in a) >= 1 and max(r.batch for r in a) <= 32
     c = make_requests(10, 1.0, seed=5, all_at_once=True)
     assert all(r.arrival == 0.0 for r in c)
+
+
+def test_tick_parts_fill_the_workspace():
+    """A tick is split by what its grouped calls need together, not by the sum of
+    what its layers would need alone."""
+    from types import SimpleNamespace
+
+    import synth
+    from paper_2311_04406_gb300 import abi, build
+    from paper_2311_04406_gb300.serve import Server
+    build.build()
+    abi.load()
+    for ring, shape in ((synth.Z64, (2048, 1024, 4096)), (synth.Z128, (512, 512, 512))):
+        L = abi.make_layer(*shape, ring.k, ring.s)
+        size = lambda n: abi.mpc_workspace_size_grouped([L] * n, abi.MPC_WS_SHARE)      # noqa: E731
+        srv = Server.__new__(Server)
+        srv.ring, srv.party, srv.nparties, srv.tag, srv._ws_cache = ring, 0, 2, "full", {}
+        srv.ws = SimpleNamespace(numel=lambda: size(8))
+        d = dict(layer=L, ws_need=srv._layer_ws(*shape))
+        reqs = [SimpleNamespace(nxt=0, bufs=[d]) for _ in range(19)]
+        parts, extra = srv._parts(reqs)
+        assert [len(p) for p in parts] == [8, 8, 3] and extra == 0
+        assert sum(parts, []) == reqs
+        srv.ws = SimpleNamespace(numel=lambda: size(1) - 1)      # not even one fits
+        parts, extra = srv._parts(reqs[:1])
+        assert parts == [reqs[:1]] and extra == size(1)
