@@ -69,7 +69,8 @@ enum {
     MPC_WS_CHECK_BATCHREC = 4,
     MPC_WS_PUBLIC_PRODUCT = 5,
     MPC_WS_OPTMAC_TRUNC = 6,
-    MPC_WS_SHARE_TRUNC = 7
+    MPC_WS_SHARE_TRUNC = 7,
+    MPC_WS_LEAST = 0x100         /* added to one of the above, see mpc_workspace_size */
 };
 
 /* Status codes */
@@ -410,7 +411,10 @@ int mpc_optmac_trunc(const mpc_layer *layer, int f, const uint64_t *alpha_i,
                      const uint64_t *P, uint64_t *Zf_i, uint64_t *mZf_i, void *stream);
 
 /* Bytes of workspace the call `which` (MPC_WS_*) needs for this layer; 0 for
- * an invalid layer.  A larger workspace is always accepted. */
+ * an invalid layer.  A larger workspace is always accepted.  which | MPC_WS_LEAST:
+ * what the call needs at least, without the planes of the residue path (see the
+ * launch table), several times smaller for layers that run there; the call then
+ * takes another path.  The same holds for mpc_workspace_size_grouped. */
 size_t mpc_workspace_size(const mpc_layer *layer, int which);
 
 /* Which ring-GEMM kernel mpc_linear_share / MPC_TAG_FULL use for this layer:

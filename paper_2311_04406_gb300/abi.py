@@ -13,6 +13,7 @@ shape (rows, cols) for Z_2^64 and (rows, cols, 2) for Z_2^128 (lo, hi).
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import threading
@@ -27,6 +28,7 @@ MPC_TAG_FULL, MPC_TAG_COMPACT, MPC_TAG_COMPACT_TRUNC = 0, 1, 2
 MPC_CHECK_COMPACT, MPC_CHECK_BATCHREC, MPC_CHECK_BATCHREC_SEEDED = 0, 1, 2
 (MPC_WS_SHARE, MPC_WS_TAG_FULL, MPC_WS_TAG_COMPACT, MPC_WS_CHECK_COMPACT, MPC_WS_CHECK_BATCHREC,
  MPC_WS_PUBLIC_PRODUCT, MPC_WS_OPTMAC_TRUNC, MPC_WS_SHARE_TRUNC) = range(8)
+MPC_WS_LEAST = 0x100         # added to one of them: the smallest workspace that runs the call
 
 # the functions include/mpclinear.h declares
 ABI_FUNCTIONS = ("mpc_linear_share", "mpc_linear_tag", "mpc_tag_check", "mpc_workspace_size",
@@ -254,10 +256,10 @@ def _native(fn, name, stream, *args, ws=0, alloc=None):
         load()
     try:
         s = _stream(stream)
-        w = () if alloc is None else (ws, -1) if ws is not None else alloc()
+        w = (None,) if alloc is None else (ws, -1, ws) if ws is not None else alloc()
     except (RuntimeError, AssertionError):
         return None          # no CUDA device: the general path checks the arguments first
-    r = getattr(_nat, name)(*args, *w, s)
+    r = getattr(_nat, name)(*args, *w[:-1], s)     # w[-1]: the workspace, alive until here
     if r:
         _check(fn, r)
     return r
@@ -299,26 +301,34 @@ def mpc_workspace_size(layer: mpc_layer, which: int) -> int:
 
 
 def _ws(layer, which, ws, stream=None):
+    """Address and bytes of the caller's workspace, or of one allocated for the
+    call, and the tensor that has to live until the call is launched."""
     if ws is not None:
-        return _ptr(ws), ws.numel() * ws.element_size()
-    need = mpc_workspace_size(layer, which)
-    if need == 0:
-        return None, 0
-    return _alloc_ws(need, stream)
+        return _ptr(ws), ws.numel() * ws.element_size(), ws
+    return _alloc_ws(lambda least: mpc_workspace_size(layer, which | least), stream)
 
 
-def _alloc_ws(need, stream):
-    """A workspace allocated on the call's stream, so that the caching
-    allocator orders its reuse after the call; it lives until the next call
-    that allocates one."""
+def _alloc_ws(size, stream):
+    """A workspace of size(0) bytes, or size(MPC_WS_LEAST) where that does not
+    fit, allocated on the call's stream, so that the caching allocator orders its
+    reuse after the call.  The allocator does not know a stream given by its
+    handle: such a call's workspace lives until the next such call."""
     import torch
-    if stream is None or isinstance(stream, int):
-        buf = torch.empty(need, dtype=torch.uint8, device="cuda")
-    else:
-        with torch.cuda.stream(stream):
+    need = size(0)
+    if need == 0:
+        return None, 0, None
+    on = contextlib.nullcontext() if stream is None or isinstance(stream, int) else torch.cuda.stream(stream)
+    with on:
+        try:
             buf = torch.empty(need, dtype=torch.uint8, device="cuda")
-    _alloc_ws.keep = buf
-    return buf.data_ptr(), need
+        except torch.cuda.OutOfMemoryError:
+            need = size(MPC_WS_LEAST)
+            if need == 0:
+                return None, 0, None
+            buf = torch.empty(need, dtype=torch.uint8, device="cuda")
+    if isinstance(stream, int):
+        _alloc_ws.keep = buf
+    return buf.data_ptr(), need, buf
 
 
 def mpc_linear_share(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None):
@@ -327,7 +337,7 @@ def mpc_linear_share(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None):
         return Z_i
     a = _args("mpc_linear_share", layer, _share_elems(layer.M, layer.K, layer.N),
               dict(E=E, F=F, A_i=A_i, B_i=B_i, C_i=C_i, Z_i=Z_i))
-    wp, wb = _ws(layer, MPC_WS_SHARE, ws, stream)
+    wp, wb, _hold = _ws(layer, MPC_WS_SHARE, ws, stream)
     _check("mpc_linear_share", load().mpc_linear_share(ctypes.byref(layer), *a, wp, wb, _stream(stream)))
     return Z_i
 
@@ -341,7 +351,7 @@ def mpc_linear_tag(layer, mode, alpha_i, E, F, mA_i, mB_i, mC_i, mZ_i, mR_i=None
     a = _args("mpc_linear_tag", layer, _tag_elems(layer.M, layer.K, layer.N, mode),
               dict(alpha_i=alpha_i, E=E, F=F, mA_i=mA_i, mB_i=mB_i, mC_i=mC_i, mR_i=mR_i, Dtilde=Dtilde,
                    chi=chi, mZ_i=mZ_i, mDc_i=mDc_i, Dc=Dc))
-    wp, wb = _ws(layer, which, ws, stream)
+    wp, wb, _hold = _ws(layer, which, ws, stream)
     _check("mpc_linear_tag", load().mpc_linear_tag(ctypes.byref(layer), int(mode), *a, wp, wb,
                                                    _stream(stream)))
     return mZ_i
@@ -359,7 +369,7 @@ def mpc_tag_check(layer, mode, alpha_i, chi_hat, opened, tag_i, cs_i, ws=None, s
         else _sized(fn, "chi_hat", chi_hat, n, w)
     a = [_sized(fn, "alpha_i", alpha_i, 1, w), ch, _sized(fn, "opened", opened, n, w),
          _sized(fn, "tag_i", tag_i, n, w), _sized(fn, "cs_i", cs_i, 1, w)]
-    wp, wb = _ws(layer, which, ws, stream)
+    wp, wb, _hold = _ws(layer, which, ws, stream)
     _check(fn, load().mpc_tag_check(ctypes.byref(layer), int(mode), *a, wp, wb, _stream(stream)))
     return cs_i
 
@@ -383,7 +393,7 @@ def mpc_linear_share_trunc(layer, E, F, A_i, B_i, C_i, Z_i, ws=None, stream=None
         return Z_i
     a = _args("mpc_linear_share_trunc", layer, _share_elems(layer.M, layer.K, layer.N),
               dict(E=E, F=F, A_i=A_i, B_i=B_i, C_i=C_i, Z_i=Z_i))
-    wp, wb = _ws(layer, MPC_WS_SHARE_TRUNC, ws, stream)
+    wp, wb, _hold = _ws(layer, MPC_WS_SHARE_TRUNC, ws, stream)
     _check("mpc_linear_share_trunc", load().mpc_linear_share_trunc(ctypes.byref(layer), *a, wp, wb,
                                                                    _stream(stream)))
     return Z_i
@@ -396,7 +406,7 @@ def mpc_public_product(layer, E, F, P, ws=None, stream=None):
         return P
     M, K, N = layer.M, layer.K, layer.N
     a = _args("mpc_public_product", layer, dict(E=M * K, F=K * N, P=M * N), dict(E=E, F=F, P=P))
-    wp, wb = _ws(layer, MPC_WS_PUBLIC_PRODUCT, ws, stream)
+    wp, wb, _hold = _ws(layer, MPC_WS_PUBLIC_PRODUCT, ws, stream)
     _check("mpc_public_product", load().mpc_public_product(ctypes.byref(layer), *a, wp, wb, _stream(stream)))
     return P
 
@@ -543,11 +553,8 @@ def mpc_launch_count_grouped(layers, which: int) -> int:
 
 def _ws_grouped(layers, which, ws, stream=None):
     if ws is not None:
-        return _ptr(ws), ws.numel() * ws.element_size()
-    need = mpc_workspace_size_grouped(layers, which)
-    if need == 0:
-        return None, 0
-    return _alloc_ws(need, stream)
+        return _ptr(ws), ws.numel() * ws.element_size(), ws
+    return _alloc_ws(lambda least: mpc_workspace_size_grouped(layers, which | least), stream)
 
 
 def mpc_linear_share_grouped(layers, ptrs, ws=None, stream=None):
@@ -557,7 +564,7 @@ def mpc_linear_share_grouped(layers, ptrs, ws=None, stream=None):
                alloc=lambda: _ws_grouped(layers, MPC_WS_SHARE, None, stream)) is not None:
         return
     pa = _ptr_array(mpc_share_ptrs, SHARE_PTR_FIELDS, ptrs, fn, layers, lambda L: _share_elems(L.M, L.K, L.N))
-    wp, wb = _ws_grouped(layers, MPC_WS_SHARE, ws, stream)
+    wp, wb, _hold = _ws_grouped(layers, MPC_WS_SHARE, ws, stream)
     _check(fn, load().mpc_linear_share_grouped(_layer_array(layers), len(layers), pa, wp, wb, _stream(stream)))
 
 
@@ -569,7 +576,7 @@ def mpc_linear_tag_grouped(layers, mode, ptrs, ws=None, stream=None):
                alloc=lambda: _ws_grouped(layers, which, None, stream)) is not None:
         return
     pa = _ptr_array(mpc_tag_ptrs, TAG_PTR_FIELDS, ptrs, fn, layers, lambda L: _tag_elems(L.M, L.K, L.N, mode))
-    wp, wb = _ws_grouped(layers, which, ws, stream)
+    wp, wb, _hold = _ws_grouped(layers, which, ws, stream)
     _check(fn, load().mpc_linear_tag_grouped(_layer_array(layers), len(layers), int(mode), pa, wp, wb,
                                              _stream(stream)))
 

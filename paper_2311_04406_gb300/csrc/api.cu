@@ -58,9 +58,9 @@ int cuda_status(cudaError_t e) {
 // run the shape, so that any launch-table choice of those tiles fits the same
 // workspace, and the residue planes of shapes near or inside that path's rule or
 // with a table entry that names it.
-size_t gemm_ws(const mpc_layer* L, int one_half = 0) {
+size_t gemm_ws(const mpc_layer* L, bool least, int one_half = 0) {
     size_t b = mpcl::gemm_tc_workspace(L->M, L->K, L->N, L->ring.words, one_half);
-    if (mpcl::gemm_crt_sized(L->M, L->K, L->N, L->ring.words))
+    if (!least && mpcl::gemm_crt_sized(L->M, L->K, L->N, L->ring.words))
         b = std::max(b, mpcl::gemm_crt_workspace(L->M, L->K, L->N, L->ring.words, one_half));
     return b;
 }
@@ -164,11 +164,12 @@ const char* mpc_status_str(int s) {
 size_t mpc_workspace_size(const mpc_layer* L, int which) {
     if (check_layer(L) != MPC_OK) return 0;
     const int w = L->ring.words;
-    switch (which) {
+    const bool least = (which & MPC_WS_LEAST) != 0;
+    switch (which & ~MPC_WS_LEAST) {
         case MPC_WS_SHARE:
         case MPC_WS_SHARE_TRUNC:
-        case MPC_WS_TAG_FULL: return gemm_ws(L);
-        case MPC_WS_PUBLIC_PRODUCT: return gemm_ws(L, 1);
+        case MPC_WS_TAG_FULL: return gemm_ws(L, least);
+        case MPC_WS_PUBLIC_PRODUCT: return gemm_ws(L, least, 1);
         case MPC_WS_OPTMAC_TRUNC: return 0;
         case MPC_WS_TAG_COMPACT: return mpcl::compact_workspace(L->M, L->K, L->N, w);
         case MPC_WS_CHECK_COMPACT: return 0;
@@ -457,7 +458,7 @@ size_t group_digit_ws(const mpc_layer* layers, int count) {
 size_t group_gemm_ws(const mpc_layer* layers, int count) {
     size_t t = group_digit_ws(layers, count);
     for (int i = 0; i < count; ++i)
-        if (layers[i].M > 0 && layers[i].N > 0) t = std::max(t, gemm_ws(&layers[i]));
+        if (layers[i].M > 0 && layers[i].N > 0) t = std::max(t, gemm_ws(&layers[i], false));
     return t;
 }
 
@@ -654,9 +655,10 @@ size_t mpc_workspace_size_grouped(const mpc_layer* layers, int count, int which)
     for (int i = 0; i < count; ++i) {
         if (check_layer(&layers[i]) != MPC_OK || !same_ring(layers[i].ring, layers[0].ring)) return 0;
     }
-    switch (which) {
+    switch (which & ~MPC_WS_LEAST) {
         case MPC_WS_SHARE:
-        case MPC_WS_TAG_FULL: return group_gemm_ws(layers, count);
+        case MPC_WS_TAG_FULL:
+            return which & MPC_WS_LEAST ? group_digit_ws(layers, count) : group_gemm_ws(layers, count);
         case MPC_WS_TAG_COMPACT: return group_compact_ws(layers, count);
         default: return 0;
     }

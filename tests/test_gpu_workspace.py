@@ -113,3 +113,61 @@ def test_residue_layers_share_their_planes(lib, ring, shapes):
         for Z, w, s in zip(Zs, want, shapes):
             assert np.array_equal(host(Z), w), (nbytes, s)
     assert abi.mpc_device_status() == 0
+
+
+def test_binding_falls_back_to_the_least_workspace(lib, monkeypatch):
+    """A workspace allocated by the binding: the residue planes where they fit, what
+    the other paths need where they do not; nothing is kept after the call."""
+    import torch
+    L = abi.make_layer(2048, 1024, 4096)
+    full = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE)
+    least = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE | abi.MPC_WS_LEAST)
+    assert 0 < least < full // 4
+    G = [L, abi.make_layer(*ODD)]
+    assert abi.mpc_workspace_size_grouped(G, abi.MPC_WS_SHARE) == full
+    assert abi.mpc_workspace_size_grouped(G, abi.MPC_WS_SHARE | abi.MPC_WS_LEAST) == least
+    for which in (abi.MPC_WS_TAG_COMPACT, abi.MPC_WS_CHECK_BATCHREC):        # one size
+        assert abi.mpc_workspace_size(L, which | abi.MPC_WS_LEAST) == abi.mpc_workspace_size(L, which)
+
+    limit, asked = full, []
+    abi._alloc_ws.__dict__.pop("keep", None)
+
+    def empty(n, dtype=None, device=None):
+        asked.append(n)
+        if n > limit:
+            raise torch.cuda.OutOfMemoryError("out of memory")
+        return torch.zeros(1)
+    monkeypatch.setattr(torch, "empty", empty)
+    assert abi._ws(L, abi.MPC_WS_SHARE, None)[1] == full
+    limit = full - 1
+    assert abi._ws(L, abi.MPC_WS_SHARE, None)[1] == least
+    assert abi._ws_grouped(G, abi.MPC_WS_SHARE, None)[1] == least
+    assert asked == [full, full, least, full, least]
+    limit = 0
+    assert abi._ws(abi.make_layer(*ODD), abi.MPC_WS_SHARE, None) == (None, 0, None)     # integer pipes
+    with pytest.raises(torch.cuda.OutOfMemoryError):
+        abi._ws(L, abi.MPC_WS_SHARE, None)
+    assert not hasattr(abi._alloc_ws, "keep")
+
+
+@pytest.mark.gpu
+def test_share_runs_where_only_the_digit_planes_fit(lib):
+    import torch
+    M, K, N = 2048, 1024, 4096
+    L = abi.make_layer(M, K, N)
+    u = lambda tid, *s: dev(synth.uniform(M + N, tid, 0, s, 64))     # noqa: E731
+    x = (u(1, M, K), u(2, K, N), u(3, M, K), u(4, K, N), u(5, M, N))
+    Z = [empty_like_ring((M, N), 1) for _ in range(2)]
+    abi.mpc_linear_share(L, *x, Z[0])
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    room = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE | abi.MPC_WS_LEAST) + (64 << 20)
+    try:
+        torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + room) / total)
+        abi.mpc_linear_share(L, *x, Z[1])
+        torch.cuda.synchronize()
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert np.array_equal(host(Z[0]), host(Z[1]))
+    assert abi.mpc_device_status() == 0
