@@ -184,8 +184,6 @@ int mpc_autotune(const mpc_layer* layers, int count, void* stream) {
                 if (!mpcl::gemm_tc_feasible(M, K, N, w, rows)) continue;
                 for (int gm : {1, 4, 8, 16}) cands.push_back(mpcl::Choice{1, gm, 0, 1, rows});
             }
-        const bool crt = mpcl::gemm_crt_candidate(M, K, N, w);
-        if (crt) cands.push_back(mpcl::Choice{1, 1, 0, 1, mpcl::CRT_TILE_ROWS, 1});
         // the integer pipes are far slower on large products: not timed there;
         // their tile height (64 or 16 rows) matters only above M = 8
         if (!tc || macs < 2147483648.0)
@@ -196,15 +194,24 @@ int mpc_autotune(const mpc_layer* layers, int count, void* stream) {
         // operands (contents do not matter for the time: every path is exact)
         const size_t e = 8 * (size_t)w;
         const size_t b_mk = e * (size_t)(M * K), b_kn = e * (size_t)(K * N), b_mn = e * (size_t)(M * N);
-        size_t ws_bytes = tc ? mpcl::gemm_tc_workspace(M, K, N, w) : 0;
-        if (crt) ws_bytes = std::max(ws_bytes, mpcl::gemm_crt_workspace(M, K, N, w));
+        const size_t digits = tc ? mpcl::gemm_tc_workspace(M, K, N, w) : 0;
+        bool crt = mpcl::gemm_crt_candidate(M, K, N, w);
+        size_t ws_bytes = crt ? std::max(digits, mpcl::gemm_crt_workspace(M, K, N, w)) : digits;
         void *E = nullptr, *X = nullptr, *B = nullptr, *F = nullptr, *C = nullptr, *Z = nullptr, *ws = nullptr;
         bool alloc = cudaMalloc(&E, b_mk > 0 ? b_mk : 16) == cudaSuccess &&
                      cudaMalloc(&X, b_mk > 0 ? b_mk : 16) == cudaSuccess &&
                      cudaMalloc(&B, b_kn > 0 ? b_kn : 16) == cudaSuccess &&
                      cudaMalloc(&F, b_kn > 0 ? b_kn : 16) == cudaSuccess &&
-                     cudaMalloc(&C, b_mn) == cudaSuccess && cudaMalloc(&Z, b_mn) == cudaSuccess &&
-                     (ws_bytes == 0 || cudaMalloc(&ws, ws_bytes) == cudaSuccess);
+                     cudaMalloc(&C, b_mn) == cudaSuccess && cudaMalloc(&Z, b_mn) == cudaSuccess;
+        if (alloc && crt && cudaMalloc(&ws, ws_bytes) != cudaSuccess) {
+            // no memory for the residue planes: the other candidates are timed
+            cudaGetLastError();
+            ws = nullptr;
+            ws_bytes = digits;
+            crt = false;
+        }
+        if (alloc && !ws && ws_bytes > 0) alloc = cudaMalloc(&ws, ws_bytes) == cudaSuccess;
+        if (crt) cands.push_back(mpcl::Choice{1, 1, 0, 1, mpcl::CRT_TILE_ROWS, 1});
         if (alloc) {
             cudaMemsetAsync(E, 0, b_mk, st);
             cudaMemsetAsync(X, 0, b_mk, st);

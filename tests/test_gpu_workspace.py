@@ -171,3 +171,25 @@ def test_share_runs_where_only_the_digit_planes_fit(lib):
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert np.array_equal(host(Z[0]), host(Z[1]))
     assert abi.mpc_device_status() == 0
+
+
+@pytest.mark.gpu
+def test_autotune_without_room_for_the_residue_planes(lib):
+    """The residue candidate is left out, and the layer is tuned among the others."""
+    import torch
+    M, K, N = 2048, 1024, 4096
+    L = abi.make_layer(M, K, N)
+    assert abi.mpc_autotune([L]) == 1 and abi.mpc_autotune_choice(L)[4] == 256     # with room
+    abi.mpc_autotune_clear()
+    operands = 8 * (2 * M * K + 2 * K * N + 2 * M * N)
+    room = operands + abi.mpc_workspace_size(L, abi.MPC_WS_SHARE | abi.MPC_WS_LEAST) + (256 << 20)
+    assert room < operands + abi.mpc_workspace_size(L, abi.MPC_WS_SHARE)
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    try:
+        assert abi.mpc_autotune([L]) == 1
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert abi.mpc_autotune_choice(L)[0] == 1 and abi.mpc_autotune_choice(L)[4] != 256
+    abi.mpc_autotune_clear()
