@@ -250,7 +250,10 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * `swizzle` tiles per tile-order group (1-64); or path 0, the integer-pipe kernels, with tiles
  * of `tile_rows` rows (64 or 16; 0 = 16 when 64-row tiles would give fewer
  * blocks than SMs, else 64; skinny layers with M <= 8 use a GEMV whatever the
- * value) and a K-split target of `waves` x 152 blocks (0 = default).  Untuned
+ * value) and a K-split target of `waves` x 152 blocks, whose sums meet in Z by
+ * atomics (0 = the built-in rule: splits that meet in the shared memory of a
+ * thread-block cluster for small layers, else a target of 4 for skinny layers and
+ * of 2).  Untuned
  * shapes use a built-in rule (tensor cores from 2^22 ring MACs, 2^20 for
  * Z_2^128; the wide tile up to two of its row tiles, and for Z_2^128 up to
  * M = 64 when it has a work unit per SM; 64-row tiles up to M = 64, the tall tile for layers with N <= 64 and M >= 2048 (Z_2^64) or
@@ -267,7 +270,7 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * mpc_autotune: for each distinct shape of layers[count], times the
  *   candidates (128-row tiles, 64-row tiles for M <= 64, the wide tile for
  *   M <= 128, the tall tile for M >= 128, each with swizzle 1/4/8/16 on the
- *   tensor cores; the residue path; tile heights 64 and 16 with K-split 1/2/4/8
+ *   tensor cores; the residue path; tile heights 64 and 16 with K-split 0/1/2/4/8
  *   on the integer pipes, below 2^31 ring MACs) on `stream` and stores the
  *   fastest.  Synchronous;
  *   allocates and frees its own scratch operands; do not call it during

@@ -444,10 +444,12 @@ cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
     while (cs < splits && cs < MAX_CLUSTER) cs *= 2;
     if (!skinny)
         while (cs > 1 && bx * by * cs > 152) cs /= 2;
-    const bool cluster = skinny ? cs >= splits && (a.N <= GV_NARROW || bx * cs <= GV_GRID)
-                                // 48 (16): beyond three (one) slices per block more splits with
-                                // atomics are faster: 16 x 400 x 160 in Z_2^64 9.9 us as clusters, 8.5 so
-                                : tm == BM_SMALL && cs > 1 && K2 <= cs * (W == 1 ? 48 : 16);
+    // a table entry with a K-split target gets that many splits, added up by atomics
+    const bool cluster = a.simt_waves == 0 &&
+                         (skinny ? cs >= splits && (a.N <= GV_NARROW || bx * cs <= GV_GRID)
+                                 // 48 (16): beyond three (one) slices per block more splits with
+                                 // atomics are faster: 16 x 400 x 160 in Z_2^64 9.9 us as clusters, 8.5 so
+                                 : tm == BM_SMALL && cs > 1 && K2 <= cs * (W == 1 ? 48 : 16));
     const bool wide = skinny && a.N > GV_NARROW && !cluster;
     int64_t kchunk, bz;
     if (cluster) {

@@ -189,7 +189,7 @@ int mpc_autotune(const mpc_layer* layers, int count, void* stream) {
         if (!tc || macs < 2147483648.0)
             for (int rows : {64, 16}) {
                 if (rows == 16 && M <= 8) continue;
-                for (int wv : {1, 2, 4, 8}) cands.push_back(mpcl::Choice{0, 0, wv, 1, M <= 8 ? 0 : rows});
+                for (int wv : {0, 1, 2, 4, 8}) cands.push_back(mpcl::Choice{0, 0, wv, 1, M <= 8 ? 0 : rows});
             }
         // operands (contents do not matter for the time: every path is exact)
         const size_t e = 8 * (size_t)w;
