@@ -31,6 +31,9 @@
 // 64 x 128 x 64 11.1, 4.5 (Z_2^128: 17.9, 8.4); 33 x 70 x 40 9.3, 4.4; 16 x 512 x 10
 // 11.2, 6.0; 8 x 299 x 368 12.4, 8.0 (18.5, 10.0); 16 x 50000 x 10 57.9, 25.9.
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -71,9 +74,8 @@ __device__ __forceinline__ typename Elem<W>::T coef_value(const GemmArgs& a) {
     return 0;
 }
 
-// The blocks of a cluster (all of grid.z of one output tile, or a group of it)
-// have written their sums of the same `count` outputs to `part` in their own
-// shared memory: block r adds up one contiguous share of the outputs over the
+// The blocks of a cluster (all of grid.z of one output tile) have written their
+// sums of the same `count` outputs to `part` in their own shared memory: block r adds up one contiguous share of the outputs over the
 // cluster and passes each sum to out(index, sum).
 template <int W, typename Out>
 __device__ __forceinline__ void cluster_sums(const typename Elem<W>::T* part, int count, Out out) {
@@ -425,8 +427,39 @@ template <int W, int VEC> Kernel gemv_kernel(int64_t M, bool wide) {
                     : ring_gemv_kernel<W, VEC, 8>;
 }
 
+// Whether the device places clusters of MAX_CLUSTER blocks of `kernel`, a size that
+// is not portable (a partition of the SMs may hold none): asked once per device and
+// kernel, together with the kernel's leave to have them.
+bool places_max_cluster(Kernel kernel) {
+    static std::mutex mu;
+    static std::map<std::pair<Kernel, int>, bool> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = known.find({kernel, dev});
+    if (it != known.end()) return it->second;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, 1, MAX_CLUSTER);
+    cfg.blockDim = dim3(NT);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = MAX_CLUSTER;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, (const void*)kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();          // the portable size serves
+        return false;
+    }
+    return known[{kernel, dev}] = n > 0;
+}
+
+// `most`: the largest cluster
 template <int W>
-cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
+cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent, int most = MAX_CLUSTER) {
     const int64_t K2 = a.one_half ? a.K : 2 * a.K;
     const bool skinny = a.M <= GV_M;
     const int vec = (skinny && W == 1 && a.N % 2 == 0) ? 2 : 1;
@@ -441,7 +474,7 @@ cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
     int64_t splits = (K2 + least - 1) / least;
     if (skinny && a.N <= GV_NARROW) splits = std::min(splits, std::max<int64_t>(1, waves * 152 / bx));
     int cs = 1;
-    while (cs < splits && cs < MAX_CLUSTER) cs *= 2;
+    while (cs < splits && cs < most) cs *= 2;
     if (!skinny)
         while (cs > 1 && bx * by * cs > 152) cs /= 2;
     // a table entry with a K-split target gets that many splits, added up by atomics
@@ -464,6 +497,10 @@ cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
         bz = K2 > 0 ? (K2 + kchunk - 1) / kchunk : 1;
     }
     if (bz > 65535) return cudaErrorInvalidConfiguration;
+    const Kernel kernel = !skinny     ? (a.N <= 16 ? tile_kernel<W, 1>(tm, cluster) : tile_kernel<W, 4>(tm, cluster))
+                          : vec == 2 ? gemv_kernel<W, 3 - W>(a.M, wide)
+                                     : gemv_kernel<W, 1>(a.M, wide);
+    if (cs > PORTABLE_CLUSTER && !places_max_cluster(kernel)) return run<W>(a, st, dependent, PORTABLE_CLUSTER);
     const int atomic = bz > cs ? 1 : 0;
     if (atomic) {
         const size_t bytes = (size_t)a.M * a.N * 8 * W;
@@ -472,13 +509,6 @@ cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent) {
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((unsigned)bx, (unsigned)by, (unsigned)bz);
-    const Kernel kernel = !skinny     ? (a.N <= 16 ? tile_kernel<W, 1>(tm, cluster) : tile_kernel<W, 4>(tm, cluster))
-                          : vec == 2 ? gemv_kernel<W, 3 - W>(a.M, wide)
-                                     : gemv_kernel<W, 1>(a.M, wide);
-    if (cs > PORTABLE_CLUSTER) {
-        const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(NT);
