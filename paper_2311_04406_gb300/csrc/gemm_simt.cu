@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "common.cuh"
@@ -75,28 +76,31 @@ __device__ __forceinline__ typename Elem<W>::T coef_value(const GemmArgs& a) {
 }
 
 // The blocks of a cluster (all of grid.z of one output tile) have written their
-// sums of the same `count` outputs to `part` in their own shared memory: block r adds up one contiguous share of the outputs over the
-// cluster and passes each sum to out(index, sum).
-template <int W, typename Out>
-__device__ __forceinline__ void cluster_sums(const typename Elem<W>::T* part, int count, Out out) {
+// sums of the same `count` outputs to `part` in their own shared memory: block r
+// adds up one contiguous share of the outputs over the cluster and stores it in Z
+// with the addend.  at(index): the output's place, or -1.
+template <int W, typename At>
+__device__ __forceinline__ void cluster_sums(const GemmArgs& a, const typename Elem<W>::T* part, int count, At at) {
     using T = typename Elem<W>::T;
     const int cs = (int)ptx::cluster_size(), rank = (int)ptx::cluster_rank();
-    __syncwarp();
-    ptx::cluster_sync();        // every block's sums are written
     const int per = (count + cs - 1) / cs;
     const int end = min(count, (rank + 1) * per);
+    __syncwarp();
+    ptx::cluster_sync();        // every block's sums are written
     for (int i = rank * per + (int)threadIdx.x; i < end; i += NT) {
+        const int64_t e = at(i);
+        const T c = e >= 0 && a.C ? ld_elem<W>(a.C, e) : (T)0;
         T s = 0;
 #pragma unroll 4
         for (int r = 0; r < cs; ++r) {
-            const uint32_t at = ptx::cluster_addr(part + i, (uint32_t)r);
+            const uint32_t p = ptx::cluster_addr(part + i, (uint32_t)r);
             if constexpr (W == 1) {
-                s += ptx::ld_cluster_u64(at);
+                s += ptx::ld_cluster_u64(p);
             } else {
-                s += (T)ptx::ld_cluster_u64(at) | ((T)ptx::ld_cluster_u64(at + 8) << 64);
+                s += (T)ptx::ld_cluster_u64(p) | ((T)ptx::ld_cluster_u64(p + 8) << 64);
             }
         }
-        out(i, s);
+        if (e >= 0) st_elem<W>(a.Z, e, s + c);
     }
     __syncwarp();
     ptx::cluster_sync();        // and read, before a block leaves
@@ -207,9 +211,9 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
     if constexpr (CLUSTER) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) Rs[ty][tx + 16 * j] = acc[0][j];
-        cluster_sums<W>(&Rs[0][0], BM_SMALL * BN, [&](int i, T v) {
+        cluster_sums<W>(a, &Rs[0][0], BM_SMALL * BN, [&](int i) {
             const int64_t m = m0 + i / BN, n = n0 + i % BN;
-            if (m < M && n < N) put<W>(a, m * N + n, v + addend<W>(a, m * N + n, 0), 0);
+            return m < M && n < N ? m * N + n : (int64_t)-1;
         });
     } else {
         auto each = [&](auto f) {
@@ -228,11 +232,63 @@ __global__ void __launch_bounds__(NT) ring_gemm_simt_kernel(GemmArgs a, int64_t 
     }
 }
 
+// acc += the left operand's staged rows times rows `first`, first + STEP, ... below
+// kc of a K chunk of [B ; F] that starts at row k0, at columns n .. n + VEC - 1.
+// The loads of U rows are in flight together; in Z_2^128 with more than two rows of
+// the left operand, which is bound by its multiply-adds, the compiler's own order
+// is as good (shares, us, with one and the other: 8 x 4608 x 512 53.1, 52.0;
+// 2 x 4096 x 4096 112, 162; Z_2^64: 3 x 1832 x 632 17.6, 22.3).  PRED: the last
+// batch of a chunk too, with zeros past its end (Ls is zero there).
+template <int W, int VEC, int MM, int STEP, bool PRED>
+__device__ __forceinline__ void gemv_rows(const GemmArgs& a, const typename Elem<W>::T* Ls, int64_t k0, int first,
+                                          int kc, int64_t n, typename Elem<W>::T (&acc)[MM][VEC]) {
+    using T = typename Elem<W>::T;
+    constexpr int U = W == 2 && MM > 2 ? 1 : 8 / W;
+    static_assert(!PRED || GV_KC % (U * STEP) == 0, "whole batches");
+    int k1 = first;
+    auto rows = [&](auto count) {
+        constexpr int B = decltype(count)::value;
+        T r[B][VEC];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int64_t kv = k0 + k1 + u * STEP;
+            const u64* row = kv < a.K ? a.B + kv * a.N * W : a.F + (kv - a.K) * a.N * W;
+            if constexpr (VEC == 2) {
+                ulonglong2 v = make_ulonglong2(0, 0);
+                if (!PRED || k1 + u * STEP < kc) v = *reinterpret_cast<const ulonglong2*>(row + n);
+                r[u][0] = v.x;
+                r[u][1] = v.y;
+            } else {
+                r[u][0] = ld_elem<W>(row, n);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+#pragma unroll
+            for (int i = 0; i < MM; ++i)
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) acc[i][v] += Ls[i * GV_KC + k1 + u * STEP] * r[u][v];
+    };
+    if constexpr (U > 1) {
+#pragma unroll 1
+        for (; k1 + (PRED ? 0 : (U - 1) * STEP) < kc; k1 += U * STEP) rows(std::integral_constant<int, U>());
+#pragma unroll 1
+        for (; k1 < kc; k1 += STEP) rows(std::integral_constant<int, 1>());
+    } else {
+#pragma unroll 8
+        for (; k1 < kc; k1 += STEP) rows(std::integral_constant<int, 1>());
+    }
+}
+
 // GEMV for wide layers: one thread per VEC output columns keeps M sums over
 // every row of the block's K range (deep independent loads along K).  VEC = 2:
 // two adjacent Z_2^64 columns per thread, read as one 16-byte vector (needs
-// even N); VEC = 1 otherwise.  MM >= M rows are accumulated (1, 2, 4 or 8).
-template <int W, int VEC, int MM>
+// even N); VEC = 1 otherwise.  MM >= M rows are accumulated (1, 2, 4 or 8).  PRED
+// (one row, Z_2^64): 30 registers in place of 48 and eight blocks per SM, faster by
+// itself (1 x 4096 x 4096 42.6, 43.8 us; 1 x 512 x 2048 5.9, 6.7) but not beside
+// the tensor-core kernels of a group, whose SMs it fills (VGG-16 at batch 1 329,
+// 311 us).
+template <int W, int VEC, int MM, bool PRED>
 __global__ void __launch_bounds__(NT) ring_gemv_wide_kernel(GemmArgs a, int64_t kchunk, int atomic) {
     using T = typename Elem<W>::T;
     __shared__ T Ls[MM][GV_KC];
@@ -257,25 +313,7 @@ __global__ void __launch_bounds__(NT) ring_gemv_wide_kernel(GemmArgs a, int64_t 
             Ls[mm][kk] = (mm < M && kk < kc) ? left<W>(a, c, mm, k0 + kk) : (T)0;
         }
         __syncthreads();
-        if (n < N) {
-#pragma unroll 8
-            for (int kk = 0; kk < kc; ++kk) {
-                const int64_t kv = k0 + kk + kr;
-                const u64* row = kv < K ? a.B + kv * N * W : a.F + (kv - K) * N * W;
-                T r[VEC];
-                if constexpr (VEC == 2) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + n);
-                    r[0] = v.x;
-                    r[1] = v.y;
-                } else {
-                    r[0] = ld_elem<W>(row, n);
-                }
-#pragma unroll
-                for (int i = 0; i < MM; ++i)
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) acc[i][v] += Ls[i][kk] * r[v];
-            }
-        }
+        if (n < N) gemv_rows<W, VEC, MM, 1, PRED>(a, &Ls[0][0], k0 + kr, 0, kc, n, acc);
         __syncthreads();
     }
     auto each = [&](auto f) {
@@ -324,25 +362,7 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
             Ls[mm][kk] = (mm < M && kk < kc) ? left<W>(a, c, mm, k0 + kk) : (T)0;
         }
         __syncthreads();
-        if (n < N) {
-#pragma unroll 8
-            for (int kk = warp; kk < kc; kk += NW) {
-                const int64_t kv = k0 + kk + kr;
-                const u64* row = kv < K ? a.B + kv * N * W : a.F + (kv - K) * N * W;
-                T r[VEC];
-                if constexpr (VEC == 2) {
-                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + n);
-                    r[0] = v.x;
-                    r[1] = v.y;
-                } else {
-                    r[0] = ld_elem<W>(row, n);
-                }
-#pragma unroll
-                for (int i = 0; i < MM; ++i)
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) acc[i][v] += Ls[i][kk] * r[v];
-            }
-        }
+        if (n < N) gemv_rows<W, VEC, MM, NW, false>(a, &Ls[0][0], k0 + kr, warp, kc, n, acc);
         __syncthreads();
     }
     if (warp > 0) {
@@ -378,10 +398,10 @@ __global__ void __launch_bounds__(NT) ring_gemv_kernel(GemmArgs a, int64_t kchun
         }
     }
     if (ptx::cluster_size() == 1) return;
-    cluster_sums<W>(part, MM * NCOL, [&](int i, T v) {
+    cluster_sums<W>(a, part, MM * NCOL, [&](int i) {
         const int row = i / NCOL;
         const int64_t col = (int64_t)blockIdx.x * NCOL + i % NCOL;
-        if (row < M && col < N) put<W>(a, row * N + col, v + addend<W>(a, row * N + col, 0), 0);
+        return row < M && col < N ? row * N + col : (int64_t)-1;
     });
 }
 
@@ -415,12 +435,12 @@ template <int W, int J> Kernel tile_kernel(int tm, bool cluster) {
     return cluster ? ring_gemm_simt_kernel<W, BM_SMALL, true, J> : ring_gemm_simt_kernel<W, BM_SMALL, false, J>;
 }
 
-template <int W, int VEC> Kernel gemv_kernel(int64_t M, bool wide) {
+template <int W, int VEC> Kernel gemv_kernel(int64_t M, bool wide, bool alone) {
     if (wide)
-        return M <= 1   ? ring_gemv_wide_kernel<W, VEC, 1>
-               : M <= 2 ? ring_gemv_wide_kernel<W, VEC, 2>
-               : M <= 4 ? ring_gemv_wide_kernel<W, VEC, 4>
-                        : ring_gemv_wide_kernel<W, VEC, 8>;
+        return M <= 1   ? (alone ? ring_gemv_wide_kernel<W, VEC, 1, VEC == 2> : ring_gemv_wide_kernel<W, VEC, 1, false>)
+               : M <= 2 ? ring_gemv_wide_kernel<W, VEC, 2, false>
+               : M <= 4 ? ring_gemv_wide_kernel<W, VEC, 4, false>
+                        : ring_gemv_wide_kernel<W, VEC, 8, false>;
     return M <= 1   ? ring_gemv_kernel<W, VEC, 1>
            : M <= 2 ? ring_gemv_kernel<W, VEC, 2>
            : M <= 4 ? ring_gemv_kernel<W, VEC, 4>
@@ -457,7 +477,8 @@ bool places_max_cluster(Kernel kernel) {
     return known[{kernel, dev}] = n > 0;
 }
 
-// `most`: the largest cluster
+// dependent: a call by itself, launched as a dependent of the kernel before it (in
+// a group on a side stream it is not); most: the largest cluster
 template <int W>
 cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent, int most = MAX_CLUSTER) {
     const int64_t K2 = a.one_half ? a.K : 2 * a.K;
@@ -498,8 +519,8 @@ cudaError_t run(const GemmArgs& a, cudaStream_t st, bool dependent, int most = M
     }
     if (bz > 65535) return cudaErrorInvalidConfiguration;
     const Kernel kernel = !skinny     ? (a.N <= 16 ? tile_kernel<W, 1>(tm, cluster) : tile_kernel<W, 4>(tm, cluster))
-                          : vec == 2 ? gemv_kernel<W, 3 - W>(a.M, wide)
-                                     : gemv_kernel<W, 1>(a.M, wide);
+                          : vec == 2 ? gemv_kernel<W, 3 - W>(a.M, wide, dependent)
+                                     : gemv_kernel<W, 1>(a.M, wide, dependent);
     if (cs > PORTABLE_CLUSTER && !places_max_cluster(kernel)) return run<W>(a, st, dependent, PORTABLE_CLUSTER);
     const int atomic = bz > cs ? 1 : 0;
     if (atomic) {
