@@ -262,8 +262,7 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  * lower, which is for layers large in both output dimensions, from about 600 in
  * Z_2^64 and 256 in Z_2^128, provided that the call's workspace covers it -- a
  * smaller workspace that covers the other paths is accepted, whether the rule or
- * an entry names the residue path, and gives the same result).  mpc_autotune_choice reports the tile that those other paths use for
- * untuned shapes.  The table is process-wide and thread-safe; workspace
+ * an entry names the residue path, and gives the same result).  The table is process-wide and thread-safe; workspace
  * sizes do not depend on it, but for the planes of an entry that names the residue
  * path for a shape far from that rule.
  *
@@ -277,8 +276,11 @@ int mpc_launch_count_grouped(const mpc_layer *layers, int count, int which);
  *   stream capture.  Returns the number of shapes tuned, or a status.
  * mpc_autotune_set: store a choice (MPC_E_MODE if the tensor-core kernel
  *   cannot run the shape with that tile height, or a value is out of range).
- * mpc_autotune_choice: the choice a call would use now; returns 1 if it comes
- *   from the table, 0 for the built-in rule.
+ * mpc_autotune_choice: returns 1 and the shape's entry, or 0 and what the
+ *   built-in rule takes among the tiles and the integer pipes.  An untuned shape
+ *   that the rule gives to the residue path runs that choice only in a workspace
+ *   without the residue planes; mpc_gemm_path and mpc_launch_count tell what runs
+ *   in one of mpc_workspace_size() bytes.
  * mpc_autotune_save / _load: the table as text ("mpclinear-autotune 2", then
  *   "words M K N path tile_rows swizzle waves" per line; version-1 files
  *   without tile_rows load as 128-row tiles); return the number of shapes, or
@@ -420,9 +422,10 @@ int mpc_optmac_trunc(const mpc_layer *layer, int f, const uint64_t *alpha_i,
  * takes another path.  The same holds for mpc_workspace_size_grouped. */
 size_t mpc_workspace_size(const mpc_layer *layer, int which);
 
-/* Which ring-GEMM kernel mpc_linear_share / MPC_TAG_FULL use for this layer:
- * 1 = the tensor-core kernel, 0 = the integer-pipe kernel, negative = invalid
- * layer (status code).  Pure host query; launches nothing. */
+/* Which ring-GEMM kernels mpc_linear_share / MPC_TAG_FULL use for this layer in a
+ * workspace of mpc_workspace_size() bytes: 1 = tensor cores (digit tiles or the
+ * residue path), 0 = the integer pipes, negative = invalid layer (status code).
+ * Pure host query; launches nothing. */
 int mpc_gemm_path(const mpc_layer *layer);
 
 /* Number of kernels the call `which` (MPC_WS_* numbering) enqueues for this

@@ -604,7 +604,10 @@ def mpc_autotune_set(layer, path: int, swizzle: int = 8, waves: int = 0, tile_ro
 
 
 def mpc_autotune_choice(layer):
-    """(path, swizzle, waves, tuned, tile_rows) the next call for this layer shape would use."""
+    """(path, swizzle, waves, tuned, tile_rows): the shape's entry in the launch table, or (tuned false) what the
+    built-in rule takes among the digit tiles and the integer pipes.  An untuned shape that the rule gives to the
+    residue path runs that only in a workspace without the residue planes: mpc_gemm_path and mpc_launch_count
+    (3 for the residue path) tell what runs in a full one."""
     p, t, g, w = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     r = load().mpc_autotune_choice(ctypes.byref(layer), ctypes.byref(p), ctypes.byref(t), ctypes.byref(g),
                                    ctypes.byref(w))

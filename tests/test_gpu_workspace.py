@@ -193,3 +193,19 @@ def test_autotune_without_room_for_the_residue_planes(lib):
         torch.cuda.empty_cache()
     assert abi.mpc_autotune_choice(L)[0] == 1 and abi.mpc_autotune_choice(L)[4] != 256
     abi.mpc_autotune_clear()
+
+
+def test_what_the_queries_report(lib):
+    """mpc_gemm_path and mpc_launch_count tell what runs in a full workspace,
+    mpc_autotune_choice the table's entry or the rule's choice without the residue
+    path."""
+    for shape, bits, other in ((ODD, 64, (0, 0)), ((2048, 1024, 4096), 64, (1, 128)), ((512, 512, 512), 128, (1, 128))):
+        L = abi.make_layer(*shape, bits // 2, bits // 2)
+        assert abi.mpc_gemm_path(L) == 1 and abi.mpc_launch_count(L, abi.MPC_WS_SHARE) == 3
+        assert abi.mpc_autotune_choice(L)[::4] == other and not abi.mpc_autotune_choice(L)[3]
+        abi.mpc_autotune_set(L, 1, 8, 0, tile_rows=256)
+        assert abi.mpc_autotune_choice(L) == (1, 8, 0, True, 256) and abi.mpc_launch_count(L, abi.MPC_WS_SHARE) == 3
+        if bits == 128:
+            abi.mpc_autotune_set(L, 1, 8, 0, tile_rows=128)
+            assert abi.mpc_autotune_choice(L)[4] == 128 and abi.mpc_launch_count(L, abi.MPC_WS_SHARE) == 2
+        abi.mpc_autotune_clear()
