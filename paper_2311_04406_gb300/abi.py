@@ -3,8 +3,8 @@
 Argument marshalling only: torch tensors supply device pointers and the
 current CUDA stream; every step of the computation runs in the library's
 kernels.  The calls that run per layer marshal their arguments in native code
-(csrc/binding.c); ctypes is the general path, which every call that fails a
-check there takes, and which raises.  Each function has the C name and raises `MpcError` on a non-zero
+(csrc/binding.c) where that is built; ctypes is the general path, which every call
+that fails a check there takes, and which raises.  Each function has the C name and raises `MpcError` on a non-zero
 status.  If the shared library is missing, loading raises immediately: there
 is no fallback path.
 
@@ -166,12 +166,11 @@ def load(build_if_missing: bool = False):
         lib.mpc_gemm_path.restype = ctypes.c_int
         lib.mpc_version.argtypes = []
         lib.mpc_version.restype = ctypes.c_int
-        if not os.path.exists(_build.BINDING):
-            raise RuntimeError(f"{_build.BINDING} is not built; run `python -c 'import __graft_entry__ as g; g.build()'`")
-        from . import _binding
-        _binding.open(path)
-        global _nat
-        _nat = _binding
+        if os.path.exists(_build.BINDING):      # without it (no Python headers at build time) ctypes marshals
+            from . import _binding
+            _binding.open(path)
+            global _nat
+            _nat = _binding
         _lib = lib
         return lib
 
@@ -252,8 +251,10 @@ def _native(fn, name, stream, *args, ws=0, alloc=None):
     """Status of the native call `name` (raised when it is an error), or None
     when the general path has to handle the arguments.  ws: a workspace tensor
     or address, None to allocate one with alloc(), 0 for calls without one."""
-    if _nat is None:
+    if _lib is None:
         load()
+    if _nat is None:
+        return None
     try:
         s = _stream(stream)
         w = (None,) if alloc is None else (ws, -1, ws) if ws is not None else alloc()

@@ -1,5 +1,6 @@
 """Build libmpclinear.so in-tree with nvcc for sm_103a (GB300), and _binding.so,
-the native argument marshalling of abi.py, with the host compiler.
+the native argument marshalling of abi.py, with the host compiler (where Python's
+headers are installed; abi.py marshals through ctypes without it).
 
 Each .cu file is compiled to an object in parallel, then linked into one
 shared library with the CUDA runtime linked statically.  The build is skipped
@@ -51,13 +52,37 @@ def _digest(extra=()) -> str:
     return h.hexdigest()
 
 
+def binding_headers():
+    """The folder of Python.h, or None."""
+    inc = sysconfig.get_paths()["include"]
+    return inc if os.path.exists(os.path.join(inc, "Python.h")) else None
+
+
+def build_binding(headers):
+    """Compile _binding.so; without Python's headers only an older one is removed."""
+    if not headers:
+        if os.path.exists(BINDING):
+            os.remove(BINDING)
+        return
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if not cc:
+        raise RuntimeError("a C compiler is required to build the binding")
+    tmp = BINDING + f".{os.getpid()}.tmp"
+    r = subprocess.run([cc, "-O2", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"), "-I" + headers, "-o", tmp,
+                        os.path.join(CSRC, "binding.c"), "-ldl"], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"the binding does not compile:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
+
+
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     nvcc = _nvcc()
     os.makedirs(BUILD, exist_ok=True)
     stamp = os.path.join(BUILD, "libmpclinear.sha256")
     dig = _digest(extra_flags)
-    if not force and os.path.exists(LIB) and os.path.exists(BINDING) and os.path.exists(stamp) and \
-             open(stamp).read() == dig:
+    headers = binding_headers()
+    if not force and os.path.exists(LIB) and (os.path.exists(BINDING) or not headers) and \
+            os.path.exists(stamp) and open(stamp).read() == dig:
         return LIB
 
     def compile_one(src):
@@ -79,16 +104,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
-    cc = shutil.which("gcc") or shutil.which("cc")
-    if not cc:
-        raise RuntimeError("a C compiler is required to build the binding")
-    tmp = BINDING + f".{os.getpid()}.tmp"
-    r = subprocess.run([cc, "-O2", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"),
-                        "-I" + sysconfig.get_paths()["include"], "-o", tmp, os.path.join(CSRC, "binding.c"), "-ldl"],
-                       capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"the binding does not compile:\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, BINDING)
+    build_binding(headers)
     with open(stamp, "w") as fh:
         fh.write(dig)
     return LIB
