@@ -119,6 +119,15 @@ static int addrs(PyObject *const *args, int n, const int64_t *elems, int words, 
     return 1;
 }
 
+/* 1: *out is the C int; 0: not an integer of that range (the general path converts or raises) */
+static int get_int(PyObject *o, int *out) {
+    int over;
+    const long v = PyLong_Check(o) ? PyLong_AsLongAndOverflow(o, &over) : 0;
+    if (!PyLong_Check(o) || over || v < INT32_MIN || v > INT32_MAX) return 0;
+    *out = (int)v;
+    return 1;
+}
+
 static int sane(const mpc_layer *L) {   /* products below fit 64 bits; other layers take the general path */
     const int64_t lim = (int64_t)1 << 31;
     return L->M >= 0 && L->K >= 0 && L->N >= 0 && L->M <= lim && L->K <= lim && L->N <= lim;
@@ -162,8 +171,8 @@ FASTCALL(py_tag) {
     ARGS(17);
     mpc_layer L;
     if (!get_layer(args[0], &L) || !sane(&L)) Py_RETURN_NONE;
-    const int mode = (int)PyLong_AsLong(args[1]);
-    if (PyErr_Occurred()) return NULL;
+    int mode;
+    if (!get_int(args[1], &mode)) Py_RETURN_NONE;
     int64_t e[12];
     uint64_t a[12], w;
     size_t wb;
@@ -182,8 +191,8 @@ FASTCALL(py_check) {
     ARGS(10);
     mpc_layer L;
     if (!get_layer(args[0], &L) || !sane(&L)) Py_RETURN_NONE;
-    const int mode = (int)PyLong_AsLong(args[1]);
-    if (PyErr_Occurred()) return NULL;
+    int mode;
+    if (!get_int(args[1], &mode)) Py_RETURN_NONE;
     const int64_t n = mode == MPC_CHECK_COMPACT ? L.M : L.M * L.N;
     uint64_t a[5], w;
     size_t wb;
@@ -221,8 +230,8 @@ FASTCALL(py_optmac) {
     ARGS(10);
     mpc_layer L;
     if (!get_layer(args[0], &L) || !sane(&L)) Py_RETURN_NONE;
-    const int f = (int)PyLong_AsLong(args[1]);
-    if (PyErr_Occurred()) return NULL;
+    int f;
+    if (!get_int(args[1], &f)) Py_RETURN_NONE;
     const int64_t n = L.M * L.N, e[7] = {1, n, n, n, n, n, n};
     uint64_t a[7];
     const int r = addrs(args + 2, 7, e, L.ring.words, a);
@@ -411,8 +420,8 @@ FASTCALL(py_share_grouped) {
 }
 FASTCALL(py_tag_grouped) {
     ARGS(6);
-    const int mode = (int)PyLong_AsLong(args[1]);
-    if (PyErr_Occurred()) return NULL;
+    int mode;
+    if (!get_int(args[1], &mode)) Py_RETURN_NONE;
     return grouped(1, mode, args[0], args[2], args[3], args[4], STREAM(5));
 }
 FASTCALL(py_check_grouped) {
