@@ -7,7 +7,10 @@
  * without calling it when a check fails or an argument is of a form it does not
  * handle; abi.py then takes the general path, which raises.  Tensors are read
  * through their Python attributes (nbytes, is_contiguous, data_ptr), so nothing
- * here depends on torch, and nothing is kept from one call for the next.
+ * here depends on torch, and nothing is kept from one call for the next.  Reading
+ * them may run Python code (subclasses, __index__), which may change the caller's
+ * lists and dicts: every item is held while it is read, and taken with a look at
+ * the list's present length.
  *
  * Why native: a grouped call checks some hundred tensors, and in Python their
  * marshalling took longer than the kernels (a call of 48 uneven layers: 1.4 ms
@@ -70,6 +73,22 @@ static int addr(PyObject *t, int sized, wide need, uint64_t *out) {
     *out = PyLong_AsUnsignedLongLongMask(p);
     Py_DECREF(p);
     return PyErr_Occurred() ? -1 : 1;
+}
+
+/* a new reference to item i, or NULL without an error when the list has become shorter */
+static PyObject *item(PyObject *list, Py_ssize_t i) {
+    if (i >= PyList_GET_SIZE(list)) return NULL;
+    PyObject *o = PyList_GET_ITEM(list, i);
+    Py_INCREF(o);
+    return o;
+}
+/* addr() of item i of a list */
+static int item_addr(PyObject *list, Py_ssize_t i, wide need, uint64_t *out) {
+    PyObject *o = item(list, i);
+    if (!o) return 0;
+    const int r = addr(o, 1, need, out);
+    Py_DECREF(o);
+    return r;
 }
 
 static uint64_t *as_words(uint64_t a) { return (uint64_t *)(uintptr_t)a; }
@@ -251,6 +270,12 @@ static int get_ints(PyObject *const *args, int n, int64_t *v) {
     }
     return 1;
 }
+static int item_int(PyObject *list, Py_ssize_t i, int64_t *v) {
+    PyObject *o = item(list, i);
+    const int ok = o && get_ints(&o, 1, v);
+    Py_XDECREF(o);
+    return ok;
+}
 static mpc_ring ring_of(const int64_t *ks) {
     mpc_ring r = {(int32_t)ks[0], (int32_t)ks[1], (int32_t)((ks[0] + ks[1] + 63) / 64)};
     return r;
@@ -326,14 +351,13 @@ FASTCALL(py_lincomb) {
     const mpc_ring ring = ring_of(v);
     if (ring.words < 1) Py_RETURN_NONE;
     const int64_t tot = numel(args[4]);
-    if (tot < 0) return NULL;
+    if (tot < 0) GIVE_UP(PyErr_Occurred() ? -1 : 0);
     const int64_t n = tot / ring.words;
     const uint64_t *in[16];
     uint64_t o;
     for (Py_ssize_t j = 0; j < cnt; ++j) {
-        PyObject *cj = PyList_GET_ITEM(args[2], j);
-        if (!get_ints(&cj, 1, &coef[j])) Py_RETURN_NONE;
-        const int r = addr(PyList_GET_ITEM(args[3], j), 1, (wide)n * ring.words * 8, &o);
+        if (!item_int(args[2], j, &coef[j])) Py_RETURN_NONE;
+        const int r = item_addr(args[3], j, (wide)n * ring.words * 8, &o);
         if (r != 1) GIVE_UP(r);
         in[j] = as_words(o);
     }
@@ -348,11 +372,15 @@ FASTCALL(py_lincomb) {
 /* the layers of a list, or NULL */
 static mpc_layer *get_layers(PyObject *list, Py_ssize_t n) {
     mpc_layer *L = PyMem_Malloc((size_t)n * sizeof(mpc_layer));
-    for (Py_ssize_t i = 0; L && i < n; ++i)
-        if (!get_layer(PyList_GET_ITEM(list, i), &L[i]) || !sane(&L[i])) {
+    for (Py_ssize_t i = 0; L && i < n; ++i) {
+        PyObject *o = item(list, i);
+        const int ok = o && get_layer(o, &L[i]) && sane(&L[i]);
+        Py_XDECREF(o);
+        if (!ok) {
             PyMem_Free(L);
             return NULL;
         }
+    }
     return L;
 }
 
@@ -365,7 +393,9 @@ static int dict_addrs(PyObject *d, PyObject *const *keys, int n, int required, c
             if (PyErr_Occurred()) return -1;
             if (required) return 0;
         }
+        Py_XINCREF(t);
         const int r = addr(t, elems[j] >= 0, (wide)elems[j] * words * 8, &a[j]);
+        Py_XDECREF(t);
         if (r != 1) return r;
     }
     return 1;
@@ -392,7 +422,9 @@ static PyObject *grouped(int kind, int mode, PyObject *layers, PyObject *ptrs, P
             e[0] = e[4] = 1;
             e[1] = e[2] = e[3] = L[i].M;
         }
-        r = dict_addrs(PyList_GET_ITEM(ptrs, i), keys, nk, kind == 2, e, L[i].ring.words, a + i * nk);
+        PyObject *d = item(ptrs, i);
+        r = d ? dict_addrs(d, keys, nk, kind == 2, e, L[i].ring.words, a + i * nk) : 0;
+        Py_XDECREF(d);
     }
     uint64_t w = 0;
     size_t wb = 0;
@@ -440,31 +472,32 @@ FASTCALL(py_lincomb_grouped) {
     if (args[5] != Py_None && (!PyList_Check(args[5]) || PyList_GET_SIZE(args[5]) != G)) Py_RETURN_NONE;
     const mpc_ring ring = ring_of(v);
     if (ring.words < 1) Py_RETURN_NONE;
-    for (Py_ssize_t j = 0; j < cnt; ++j) {
-        PyObject *cj = PyList_GET_ITEM(args[2], j);
-        if (!get_ints(&cj, 1, &coef[j])) Py_RETURN_NONE;
-    }
+    for (Py_ssize_t j = 0; j < cnt; ++j)
+        if (!item_int(args[2], j, &coef[j])) Py_RETURN_NONE;
     uint64_t *buf = PyMem_Malloc((size_t)G * (cnt + 2) * 8);   /* ins, outs, sizes */
     if (!buf) Py_RETURN_NONE;
     uint64_t *in = buf, *out = buf + G * cnt;
     int64_t *n = (int64_t *)(out + G);
     int r = 1;
     for (Py_ssize_t g = 0; r == 1 && g < G; ++g) {
-        PyObject *o = PyList_GET_ITEM(args[4], g), *row = PyList_GET_ITEM(args[3], g);
-        if (args[5] != Py_None) {
-            PyObject *ng = PyList_GET_ITEM(args[5], g);
-            if (!get_ints(&ng, 1, &n[g])) r = 0;
+        PyObject *o = item(args[4], g), *row = item(args[3], g);
+        if (!o || !row) {
+            r = 0;
+        } else if (args[5] != Py_None) {
+            r = item_int(args[5], g, &n[g]);
         } else if (o == Py_None || PyLong_Check(o)) {
             r = 0;
         } else {
             n[g] = numel(o);
-            if (n[g] < 0) r = -1;
+            if (n[g] < 0) r = PyErr_Occurred() ? -1 : 0;
             else n[g] /= ring.words;
         }
         if (r == 1 && (!PyList_Check(row) || PyList_GET_SIZE(row) != cnt)) r = 0;
         for (Py_ssize_t j = 0; r == 1 && j < cnt; ++j)
-            r = addr(PyList_GET_ITEM(row, j), 1, (wide)n[g] * ring.words * 8, &in[g * cnt + j]);
+            r = item_addr(row, j, (wide)n[g] * ring.words * 8, &in[g * cnt + j]);
         if (r == 1) r = addr(o, 1, (wide)n[g] * ring.words * 8, &out[g]);
+        Py_XDECREF(o);
+        Py_XDECREF(row);
     }
     int status = 0;
     void *st = STREAM(6);

@@ -122,6 +122,28 @@ def test_grouped_operands_are_checked():
     assert nat.tag_grouped([L], 1.0, [{k: _Buf(8 * n) for k, n in sizes.items()}], *ws, 0) is None
 
 
+@pytest.mark.hidden_gpu
+def test_lists_that_change_while_they_are_read():
+    nat = abi._nat
+    ins = []
+    ins[:] = [_Buf(64, on_read=ins.clear), _Buf(64)]
+    assert nat.lincomb(32, 32, [1, 1], ins, _Buf(64), 0) is None
+    row = []
+    row[:] = [_Buf(64, on_read=row.clear), _Buf(64)]
+    assert nat.lincomb_grouped(32, 32, [1, 1], [row, [_Buf(64)] * 2], [_Buf(64)] * 2, None, 0) is None
+    outs = []
+    outs[:] = [_Buf(64, on_read=outs.clear), _Buf(64)]
+    assert nat.lincomb_grouped(32, 32, [1], [[_Buf(64)]] * 2, outs, None, 0) is None
+    L = abi.make_layer(2, 2, 2)
+    e = abi._share_elems(2, 2, 2)
+    ptrs = []
+    ptrs[:] = [{k: _Buf(8 * n, on_read=ptrs.clear) for k, n in e.items()}, {k: _Buf(8 * n) for k, n in e.items()}]
+    assert nat.share_grouped([L, L], ptrs, 0x100000, 1 << 30, 0) is None
+    p = {}
+    p.update({k: _Buf(8 * n, on_read=p.clear) for k, n in e.items()})
+    assert nat.share_grouped([L], [p], 0x100000, 1 << 30, 0) == abi.MPC_E_NULL      # the operands are gone
+
+
 @pytest.mark.gpu
 def test_refusals_on_the_gpu():
     """The same through the public calls: the general path raises, nothing is launched."""
