@@ -444,13 +444,14 @@ int mpc_launch_count(const mpc_layer *layer, int which);
  * device. */
 int mpc_device_status(void);
 
-/* Self-test of the bounded device-side wait (no counterpart in the paper):
+/* Self-test of the bounded device-side waits (no counterpart in the paper):
  * one thread waits on a barrier that nothing arrives at, for at most
  * limit_cycles clock cycles (1e3 .. 1e10; about 1e9 per 0.5 s at 2 GHz), then
- * gives up and records the timeout as the GEMM's roles do.  Synchronous on
- * `stream`.  Returns MPC_E_TIMEOUT when the wait gave up (the expected
- * outcome; the flag that mpc_device_status reads is then set), MPC_OK if it did
- * not, MPC_E_SHAPE for a limit out of range, MPC_E_CUDA on a CUDA error.  The
+ * gives up and records the timeout as the GEMM's roles do; first as the digit
+ * tiles, whose flag it reads, then as the residue path.  Synchronous on
+ * `stream`.  Returns MPC_E_TIMEOUT when both waits gave up and the first was
+ * reported (the expected outcome; the flag that mpc_device_status reads is then
+ * set by the second), MPC_OK if not, MPC_E_SHAPE for a limit out of range, MPC_E_CUDA on a CUDA error.  The
  * context stays usable afterwards. */
 int mpc_selftest_wait(long long limit_cycles, void *stream);
 

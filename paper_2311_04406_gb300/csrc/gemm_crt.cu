@@ -1123,4 +1123,34 @@ int crt_timeout_flag(bool* set, cudaStream_t s) {
     return 0;
 }
 
+namespace {
+__device__ int g_crt_selftest_gave_up = 0;
+
+// the wait of the pair's kernel on a barrier that nothing arrives at
+__global__ void crt_wait_selftest_kernel(long long limit) {
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ int abort_flag;
+    if (threadIdx.x == 0) {
+        ptx::mbar_init(&bar, 1);
+        abort_flag = 0;
+        ptx::fence_barrier_init();
+        g_crt_selftest_gave_up = 0;
+        if (!ptx::mbar_wait_cluster(&bar, 0, &abort_flag, limit)) {
+            gave_up(&abort_flag);
+            g_crt_selftest_gave_up = 1;
+        }
+    }
+}
+}  // namespace
+
+int crt_wait_selftest(long long limit, cudaStream_t st) {
+    int v = 0;
+    crt_wait_selftest_kernel<<<1, 32, 0, st>>>(limit);
+    if (cudaGetLastError() != cudaSuccess ||
+        cudaMemcpyFromSymbolAsync(&v, g_crt_selftest_gave_up, sizeof(v), 0, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return -1;
+    return v;
+}
+
 }  // namespace mpcl

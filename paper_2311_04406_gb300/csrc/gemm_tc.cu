@@ -2475,9 +2475,11 @@ int gemm_tc_grouped_launches(const int64_t* M, const int64_t* K, const int64_t* 
 }
 
 // ---------------------------------------------------------------------------
-// self-test of the bounded wait: one thread waits on a barrier that nothing
+// self-test of the bounded waits: one thread waits on a barrier that nothing
 // arrives at; the wait must give up after `limit` cycles and record the
-// timeout exactly as the GEMM's roles do.
+// timeout exactly as the GEMM's roles do.  First the wait and flag of this file's
+// kernels, whose flag has to be read here, then those of the residue path, whose
+// flag is left for the next status query.
 
 namespace {
 __device__ int g_selftest_gave_up = 0;
@@ -2501,7 +2503,8 @@ __global__ void wait_selftest_kernel(long long limit) {
 }
 }  // namespace
 
-int wait_selftest(long long limit, cudaStream_t st) {
+namespace {
+int run_wait_selftest(long long limit, cudaStream_t st) {
     int zero = 0, v = 0;
     if (cudaMemcpyToSymbolAsync(g_selftest_gave_up, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st) !=
         cudaSuccess)
@@ -2513,6 +2516,15 @@ int wait_selftest(long long limit, cudaStream_t st) {
         return -1;
     if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
     return v;
+}
+}  // namespace
+
+int wait_selftest(long long limit, cudaStream_t st) {
+    const int own = run_wait_selftest(limit, st);
+    bool set = false;
+    if (own < 0 || tc_timeout_flag(&set) != 0) return -1;
+    const int crt = crt_wait_selftest(limit, st);
+    return crt < 0 ? -1 : own == 1 && set && crt == 1;
 }
 
 namespace {

@@ -90,6 +90,7 @@ size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_ha
 constexpr int CRT_LAUNCHES = 3;
 cudaError_t launch_gemm_crt(const GemmArgs& a, void* ws, size_t ws_bytes, cudaStream_t st);
 int crt_timeout_flag(bool* set, cudaStream_t s);   // synchronous; 0 on success
+int crt_wait_selftest(long long limit, cudaStream_t st);   // synchronous; 1 when the wait gave up, -1 on an error
 
 // CompactTag path (a3, a4, a5)
 struct CompactArgs {

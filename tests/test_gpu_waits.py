@@ -41,3 +41,21 @@ def test_bounded_wait_gives_up_and_context_survives():
 def test_selftest_rejects_bad_limits():
     assert abi.mpc_selftest_wait(10) == abi.MPC_E_SHAPE
     assert abi.mpc_selftest_wait(10**11) == abi.MPC_E_SHAPE
+
+
+def test_each_kernel_family_reports_its_timeout():
+    """The self-test runs out the wait of the digit tiles and, after their flag has
+    been read, that of the residue path's pairs: the status that is left is the
+    latter's, once, and a layer on that path is exact afterwards."""
+    for _ in range(2):
+        assert abi.mpc_device_status() == 0
+        assert abi.mpc_selftest_wait(2_000_000) == abi.MPC_E_TIMEOUT
+        assert abi.mpc_device_status() == abi.MPC_E_TIMEOUT
+        assert abi.mpc_device_status() == 0
+    M, K, N = 300, 100, 130
+    abi.mpc_autotune_set(abi.make_layer(M, K, N), 1, tile_rows=256)
+    u = lambda t, *s: synth.uniform(4, t, 0, s, 64)     # noqa: E731
+    E, F, A, B, C = u(1, M, K), u(2, K, N), u(3, M, K), u(4, K, N), u(5, M, N)
+    assert np.array_equal(gpu_share(synth.Z64, 0, E, F, A, B, C), O.linear_share(64, 0, E, F, A, B, C))
+    abi.mpc_autotune_clear()
+    assert abi.mpc_device_status() == 0
