@@ -95,8 +95,8 @@ constexpr double product(int n) {
 }
 constexpr double pow2(int n) { return n == 0 ? 1.0 : 2.0 * pow2(n - 1); }
 constexpr int64_t CRT_MAX_K2 = int64_t(1) << 15;   // padded inner dimension 2K
-static_assert(product(16) > 3.5 * pow2(15) * pow2(126) && product(31) > 3.5 * pow2(15) * pow2(254),
-              "|V| / P stays below 0.29");
+static_assert(0.30 * product(16) > 1.13 * pow2(15) * pow2(126) && 0.30 * product(31) > 1.02 * pow2(15) * pow2(254),
+              "|V| / P stays below 0.30");
 
 // symmetric residue of a (a >= 0)
 constexpr int sym(int64_t a, int p) {
