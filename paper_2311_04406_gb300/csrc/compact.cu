@@ -221,13 +221,10 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
 }
 
 // FOLD is a template parameter: with both forms in one kernel it took 74
-// registers in place of 62, three blocks per SM in place of four, and the call
-// of a 128 x 4096 x 4096 layer 0.9 us more.  Four blocks are also asked for where
-// the compiler would take more than 64 registers in Z_2^64 (here without FOLD, and
-// in the grouped kernel: 0.3-0.4 % of a truncated 2048 x 1024 x 4096 layer, of
-// VGG-16 at batch 32 and of 48 uneven layers).
+// registers in place of 62 (now 64), three blocks per SM in place of four, and the
+// call of a 128 x 4096 x 4096 layer 0.9 us more.
 template <int W, int VEC, bool FOLD>
-__global__ void __launch_bounds__(NT, W == 1 && VEC == 2 && !FOLD ? 4 : 0) rows_kernel(RowsParams p) {
+__global__ void __launch_bounds__(NT) rows_kernel(RowsParams p) {
     ptx::grid_dep_launch();   // finalize and vec wait for this grid before reading
     ptx::grid_dep_wait();     // launched as a dependent of the kernel before it
     rows_body<W, VEC, FOLD>(p, (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5), threadIdx.x & 31);
@@ -539,7 +536,7 @@ __device__ __forceinline__ int layer_of(const int64_t* off, int count, int64_t b
 }
 
 template <int W>
-__global__ void __launch_bounds__(NT, W == 1 ? 4 : 0) rows_group_kernel(const __grid_constant__ CompactGroup g) {
+__global__ void __launch_bounds__(NT) rows_group_kernel(const __grid_constant__ CompactGroup g) {
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();
     const int li = layer_of(g.rb, g.count, blockIdx.x);
