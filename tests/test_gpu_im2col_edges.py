@@ -33,3 +33,24 @@ def test_im2col_block_edges(ring, cfg):
     out = empty_like_ring((B * Ho * Wo, C * f * f), ring.words)
     abi.mpc_im2col(ring.k, ring.s, B, C, H, W, f, pad, stride, dev(x), out)
     assert np.array_equal(host(out), O.im2col(x, f, pad, stride, ring.bits))
+
+
+@pytest.mark.gpu
+def test_im2col_of_many_small_images_costs_what_its_bytes_do():
+    """200,000 images of one value against one image of as many: the same bytes."""
+    import torch
+
+    def best(B, H, W):
+        x = torch.zeros(B * H * W, dtype=torch.int64, device="cuda")
+        out = torch.empty_like(x)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        t = []
+        for _ in range(8):
+            e[0].record()
+            for _ in range(20):
+                abi.mpc_im2col(32, 32, B, 1, H, W, 1, 0, 1, x, out)
+            e[1].record()
+            torch.cuda.synchronize()
+            t.append(e[0].elapsed_time(e[1]))
+        return min(t)
+    assert best(200000, 1, 1) < 3 * best(1, 400, 500)
