@@ -174,7 +174,8 @@ int mpc_tag_check(const mpc_layer *layer, int mode, const uint64_t *alpha_i,
  * A tensor-core layer long enough to keep every SM busy for 64 waves of units
  * gets a launch pair of its own (it gains nothing from sharing one and runs
  * faster alone).  Layers on the residue path (see the launch table) run one
- * after another: Z_2^128 layers, and Z_2^64 layers with odd N or a table entry.
+ * after another behind them; Z_2^64 layers with even N take it here up to 1 GiB of
+ * planes, or with a table entry.
  *
  * layers[count], ptrs[count]: HOST arrays, read during the call only.  All
  * layers share one ring (MPC_E_RING otherwise); the party may differ per

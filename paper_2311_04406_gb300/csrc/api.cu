@@ -60,7 +60,8 @@ int cuda_status(cudaError_t e) {
 // with a table entry that names it.
 size_t gemm_ws(const mpc_layer* L, bool least, int one_half = 0) {
     size_t b = mpcl::gemm_tc_workspace(L->M, L->K, L->N, L->ring.words, one_half);
-    if (!least && mpcl::gemm_crt_sized(L->M, L->K, L->N, L->ring.words))
+    if (!least && (mpcl::gemm_crt_near(L->M, L->K, L->N, L->ring.words) ||
+                   mpcl::gemm_crt_named(L->M, L->K, L->N, L->ring.words)))
         b = std::max(b, mpcl::gemm_crt_workspace(L->M, L->K, L->N, L->ring.words, one_half));
     return b;
 }
@@ -433,11 +434,23 @@ bool on_tc(const mpc_layer& L) {
 }
 
 // The residue path in a group: a layer there runs by itself, where the digit
-// tiles share their launches, so the rule asks for a larger gain.  Z_2^64 layers
-// that the digit tiles can run stay with them unless the table says otherwise.
+// tiles share their launches, so the rule asks for a larger gain (crt_ratio).
+// Shares of Z_2^64 groups, us, with the layers that the rule takes on the digit
+// tiles and on this path: 48 uneven layers (1129 x 1692 x 1468 of them) 842, 778;
+// the same drawn otherwise (1833 x 1292 x 1002) 894, 822; 2048 x 1024 x 4096 and
+// 2048 x 4096 x 1024 three times 5055, 3098; VGG-16 at batch 64 (1024 x 4608 x 512)
+// 2532, 2468.  Z_2^64 layers that the digit tiles can run take it with at most
+// GROUP_PLANES of planes, which bounds what a group's workspace grows by;
+// larger ones (2048 x 4096 x 4096: 1.9 GB, in place of 0.5) keep a launch pair of
+// their own on the digit tiles unless the table names the path.
+constexpr size_t GROUP_PLANES = size_t(1) << 30;
+bool group_rule(int64_t M, int64_t K, int64_t N, int words) {
+    return mpcl::gemm_crt_preferred(M, K, N, words, true) &&
+           (words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words) ||
+            mpcl::gemm_crt_workspace(M, K, N, words) <= GROUP_PLANES);
+}
 bool group_uses_crt(const mpcl::Choice& c, int64_t M, int64_t K, int64_t N, int words) {
-    if (!c.crt || c.tuned) return c.crt != 0;
-    return (words == 2 || !mpcl::gemm_tc_feasible(M, K, N, words)) && mpcl::gemm_crt_preferred(M, K, N, words, true);
+    return c.crt && (c.tuned || group_rule(M, K, N, words));
 }
 
 // Workspace of a grouped GEMM (whatever the launch table picks): the digit planes
@@ -457,8 +470,12 @@ size_t group_digit_ws(const mpc_layer* layers, int count) {
 
 size_t group_gemm_ws(const mpc_layer* layers, int count) {
     size_t t = group_digit_ws(layers, count);
-    for (int i = 0; i < count; ++i)
-        if (layers[i].M > 0 && layers[i].N > 0) t = std::max(t, gemm_ws(&layers[i], false));
+    for (int i = 0; i < count; ++i) {
+        const mpc_layer& L = layers[i];
+        if (L.M > 0 && L.N > 0 &&
+            (group_rule(L.M, L.K, L.N, L.ring.words) || mpcl::gemm_crt_named(L.M, L.K, L.N, L.ring.words)))
+            t = std::max(t, mpcl::gemm_crt_workspace(L.M, L.K, L.N, L.ring.words));
+    }
     return t;
 }
 

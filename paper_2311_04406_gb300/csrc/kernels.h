@@ -81,10 +81,10 @@ int tc_timeout_flag(bool* set);   // synchronous; 0 on success
 // ring GEMM from residue products (exact); layers large in both output
 // dimensions.  Near: shapes close to or inside the built-in rule, whose workspace
 // covers this path.  Candidate: those, and small ones, which the launch table may
-// give to it; sized: near or given to it.
+// give to it; named: given to it by the launch table.
 bool gemm_crt_near(int64_t M, int64_t K, int64_t N, int words);
 bool gemm_crt_candidate(int64_t M, int64_t K, int64_t N, int words);
-bool gemm_crt_sized(int64_t M, int64_t K, int64_t N, int words);
+bool gemm_crt_named(int64_t M, int64_t K, int64_t N, int words);
 bool gemm_crt_preferred(int64_t M, int64_t K, int64_t N, int words, bool grouped = false);
 size_t gemm_crt_workspace(int64_t M, int64_t K, int64_t N, int words, int one_half = 0);
 constexpr int CRT_LAUNCHES = 3;

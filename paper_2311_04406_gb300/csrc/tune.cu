@@ -100,8 +100,7 @@ Choice gemm_choice(int64_t M, int64_t K, int64_t N, int words) {
     return gemm_built_in(M, K, N, words);
 }
 
-bool gemm_crt_sized(int64_t M, int64_t K, int64_t N, int words) {
-    if (gemm_crt_near(M, K, N, words)) return true;
+bool gemm_crt_named(int64_t M, int64_t K, int64_t N, int words) {
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = table().find(Key{words, M, K, N});
     return it != table().end() && it->second.path == 1 && it->second.rows == CRT_TILE_ROWS;

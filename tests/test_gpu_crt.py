@@ -124,3 +124,28 @@ def test_residue_path_rule():
     assert not crt(128, 4096, 4096) and not crt(32768, 576, 64) and not crt(1024, 576, 64)
     assert not crt(8, 4096, 4096, 128) and not crt(32768, 576, 64, 128) and not crt(64, 128, 64)
     assert not crt(1024, 16385, 1024), "2K beyond the proven range"
+
+
+def test_residue_path_rule_in_groups():
+    """A group's layers take the path by its own estimate in both rings, also where
+    the digit tiles could run them."""
+    abi.mpc_autotune_clear()
+
+    def crt(M, K, N, bits):
+        Ls = [abi.make_layer(M, K, N, bits // 2, bits // 2)]
+        n = abi.mpc_launch_count_grouped(Ls * 2, abi.MPC_WS_SHARE)
+        assert n in (6, 2)      # three launches per layer, or a launch pair for both
+        return n == 6
+    assert crt(1129, 1692, 1468, 64) and crt(2048, 1024, 4096, 64) and crt(1000, 999, 1001, 64)
+    assert crt(1024, 2304, 256, 128) and crt(512, 512, 512, 128)
+    assert not crt(1024, 576, 64, 64) and not crt(128, 4096, 4096, 64) and not crt(512, 512, 512, 64)
+    # 1.9 GB of planes: a launch pair of its own on the digit tiles, and no planes in the workspace
+    big = abi.make_layer(2048, 4096, 4096)
+    assert abi.mpc_launch_count(big, abi.MPC_WS_SHARE) == 3
+    assert abi.mpc_launch_count_grouped([big], abi.MPC_WS_SHARE) == 2
+    size = abi.mpc_workspace_size_grouped([big], abi.MPC_WS_SHARE)
+    assert size == abi.mpc_workspace_size_grouped([big], abi.MPC_WS_SHARE | abi.MPC_WS_LEAST)
+    abi.mpc_autotune_set(big, 1, tile_rows=CRT)
+    assert abi.mpc_launch_count_grouped([big], abi.MPC_WS_SHARE) == 3
+    assert abi.mpc_workspace_size_grouped([big], abi.MPC_WS_SHARE) > size
+    abi.mpc_autotune_clear()
