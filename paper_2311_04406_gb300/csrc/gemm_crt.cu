@@ -29,7 +29,8 @@
 //      matrices).  Elements are split into 10-bit pieces; small warp-level MMAs
 //      multiply the pieces by 2^(10 j) mod p_i, and the sums are reduced in
 //      packed fp32.  Bound: memory (8 W bytes read, 2 NP written per element);
-//      measured 7.5 ps per element in Z_2^64 (floor 5.9), 17 in Z_2^128 (11.5).
+//      measured 7.2 ps per element in Z_2^64 (floor 5.9), 13.6 in Z_2^128 (15.6
+//      where cE is added; 11.5).
 //      With fp32 multiply-adds in place of the small MMAs Z_2^128 took 31 ps.
 //   2. residue_gemm_kernel  plain fp16 GEMMs, one per (modulus, output tile):
 //      CTA pairs (cta_group::2) on 256 x 256 tiles, because one CTA per tile
@@ -43,10 +44,10 @@
 //      output, by small MMAs again.  Bound: memory (2 NP + 16 W bytes per output).
 //
 // Share calls, digit tiles (gemm_tc.cu) -> this path, measured on GB300:
-// Z_2^64 2048 x 1024 x 4096 841 -> 519 us, 2048 x 1024 x 1024 233 -> 166 us,
-// 4096 x 4096 x 4096 6.6 -> 3.2 ms, 1000 x 999 x 1001 (odd N, integer pipes)
-// 928 -> 123 us; Z_2^128 2048 x 2304 x 256 606 -> 352 us, 512 x 4608 x 512
-// 503 -> 292 us, 512 x 512 x 512 80 -> 52 us.  Splitting the operands costs
+// Z_2^64 2048 x 1024 x 4096 841 -> 507 us, 2048 x 1024 x 1024 233 -> 158 us,
+// 4096 x 4096 x 4096 6.6 -> 3.3 ms, 1000 x 999 x 1001 (odd N, integer pipes)
+// 928 -> 115 us; Z_2^128 2048 x 2304 x 256 606 -> 331 us, 512 x 4608 x 512
+// 503 -> 274 us, 512 x 512 x 512 80 -> 46 us.  Splitting the operands costs
 // (M + N) 2K elements against 2 M N K multiply-adds, so layers with one small
 // side (128 x 4096 x 4096, convolutions with 64 outputs) stay with the digits.
 #include <cuda.h>

@@ -27,9 +27,10 @@
 // A block's time goes with its K slices (a 16-deep one takes about 1 us in
 // Z_2^64, 3-4 us in Z_2^128: the low 64 or 128 bits of a product need 1 or 6
 // wide multiply-adds, which issue at 15 per clock cycle and SM), so small layers
-// spread K over as many blocks as fit the chip once.  Shares before and now, us:
-// 64 x 128 x 64 11.1, 4.5 (Z_2^128: 17.9, 8.4); 33 x 70 x 40 9.3, 4.4; 16 x 512 x 10
-// 11.2, 6.0; 8 x 299 x 368 12.4, 8.0 (18.5, 10.0); 16 x 50000 x 10 57.9, 25.9.
+// spread K over as many blocks as fit the chip once.  Shares, us, with a copy of C
+// and atomics and now: 64 x 128 x 64 11.1, 4.4 (Z_2^128: 17.9, 8.2); 33 x 70 x 40 9.3,
+// 4.3; 16 x 512 x 10 11.2, 6.6; 8 x 299 x 368 12.4, 6.4 (18.5, 10.0); 16 x 50000 x 10
+// 57.9, 27.3.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -51,7 +52,7 @@ constexpr int GV_KC = 128;      // K chunk staged in shared memory
 constexpr int PORTABLE_CLUSTER = 8, MAX_CLUSTER = 16;
 constexpr int GV_NARROW = 256;  // N up to here: ring_gemv_kernel for any K
 constexpr int GV_GRID = 200;    // blocks up to which wider layers take it too, when their K splits fit one
-                                // cluster (measured: 4 x 512 x 1000, 128 blocks, 11.5 -> 9.1 us; 1 x 512 x 4096,
+                                // cluster (measured: 4 x 512 x 1000, 128 blocks, 11.5 -> 8.9 us; 1 x 512 x 4096,
                                 // 512 blocks, would go from 6.7 to 9.4)
 
 

@@ -1074,8 +1074,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) ring_gemm_tc_kernel(const __grid_
         // addition) leaves while the next tile is drained.  With loads and stores
         // by the warp a tile's epilogue took 11,100 clock cycles, more than the
         // MMAs of a tile with 2K = 256, and a split piece 5,800: the share of a
-        // 4096 x 128 x 4096 layer took 354 us and takes 248, of 1024 x 576 x 64
-        // 18.9 and 17.2, of 256 x 576 x 128 17.0 and 15.4.
+        // 4096 x 128 x 4096 layer took 354 us and takes 247, of 1024 x 576 x 64
+        // 18.9 and 16.9, of 256 x 576 x 128 17.0 and 14.6.
         constexpr int RPW = R / 4;      // tile rows per drain warp
         constexpr uint32_t STG_ROW = Lay::STG_ROW;
         const int quad = warp & 3;

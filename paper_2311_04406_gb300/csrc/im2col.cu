@@ -33,7 +33,7 @@ struct Im2colArgs {
 // Consecutive threads take consecutive columns, so the writes are coalesced, and
 // the reads of neighbouring rows share lines.  One thread per element with six 64-bit
 // divisions each was bound by their instructions: 1 x 64 x 32 x 32 with f = 3
-// took 7.5 us and takes 3.9, 128 such images 532 and 128 (Z_2^128: 538 and 208,
+// took 7.5 us and takes 3.8, 128 such images 532 and 127 (Z_2^128: 538 and 208,
 // 5.8 TB/s written).
 constexpr int UNROLL = 4;       // loads in flight per thread
 
