@@ -83,7 +83,8 @@ __device__ __forceinline__ void st_elem(u64* p, int64_t i, typename Elem<W>::T v
 }
 
 // 16-byte load at this point of the program (a plain one is moved about by the
-// compiler: the CompactTag rows kernel then took 76 registers in place of 62)
+// compiler: the grouped CompactTag rows kernel then takes 76 registers in place of
+// 64, the vec kernel of few rows 64 in place of 44)
 __device__ __forceinline__ ulonglong2 ld_pair(const u64* p) {
     ulonglong2 v;
     asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));

@@ -142,7 +142,7 @@ struct RowsParams {
 
 // VEC = 2: two Z_2^64 elements per 16-byte access (needs even N).  Warp
 // task g of one layer.
-template <int W, int VEC, bool FOLD>
+template <int W, int VEC, bool FOLD, bool GROUP = false>
 __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int lane) {
     using T = typename Elem<W>::T;
     const int64_t tasksA = p.M * p.S, tasksB = p.K * p.S;
@@ -159,7 +159,7 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
         const int64_t base = row * p.N;
         if constexpr (VEC == 2) {
             for (int64_t c = c0 + 2 * lane; c < c1; c += 64) {
-                ulonglong2 x = ld_pair(p.chi + c);
+                const ulonglong2 x = GROUP ? ld_pair(p.chi + c) : *reinterpret_cast<const ulonglong2*>(p.chi + c);
                 ulonglong2 r = ld_stream2(p.mR + base + c);
                 ulonglong2 d = ld_stream2(p.Dt + base + c);
                 ulonglong2 m = ld_stream2(p.mC + base + c);
@@ -197,7 +197,7 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
         const int64_t base = row * p.N;
         if constexpr (VEC == 2) {
             for (int64_t c = c0 + 2 * lane; c < c1; c += 64) {
-                ulonglong2 x = ld_pair(p.chi + c);
+                const ulonglong2 x = GROUP ? ld_pair(p.chi + c) : *reinterpret_cast<const ulonglong2*>(p.chi + c);
                 ulonglong2 b = ld_stream2(p.mB + base + c);
                 ulonglong2 f = ld_stream2(p.F + base + c);
                 s1 += b.x * x.x + b.y * x.y;
@@ -220,11 +220,15 @@ __device__ __forceinline__ void rows_body(const RowsParams& p, int64_t g, int la
     }
 }
 
-// FOLD is a template parameter: with both forms in one kernel it took 74
-// registers in place of 62 (now 64), three blocks per SM in place of four, and the
-// call of a 128 x 4096 x 4096 layer 0.9 us more.
+// FOLD is a template parameter: with both forms in one kernel it took 74 registers
+// and three blocks per SM in place of four.  Bound by the loads in flight.  On pairs
+// (Z_2^64) a bound of four blocks per SM, with chi loaded where the compiler likes
+// and 24-48 bytes per thread spilled, takes 50.2 us for the call of a
+// 128 x 4096 x 4096 layer and its check; chi's load held in place, without a bound
+// and without spills (64 registers too), 52.5.  The grouped kernel, which carries
+// both forms, is better the second way (GROUP; VGG-16 at batch 32 1694 us, 1698).
 template <int W, int VEC, bool FOLD>
-__global__ void __launch_bounds__(NT) rows_kernel(RowsParams p) {
+__global__ void __launch_bounds__(NT, W == 1 && VEC == 2 ? 4 : 0) rows_kernel(RowsParams p) {
     ptx::grid_dep_launch();   // finalize and vec wait for this grid before reading
     ptx::grid_dep_wait();     // launched as a dependent of the kernel before it
     rows_body<W, VEC, FOLD>(p, (int64_t)blockIdx.x * WARPS + (threadIdx.x >> 5), threadIdx.x & 31);
@@ -299,8 +303,8 @@ __device__ __forceinline__ void vec_body(const VecParams& p, int wpr, int64_t bl
         if constexpr (VEC == 2) {
 #pragma unroll 4
             for (int64_t k = 2 * (sub * 32 + lane); k < p.K; k += 64 * wpr) {
-                ulonglong2 e = *reinterpret_cast<const ulonglong2*>(p.E + base + k);
-                ulonglong2 ma = *reinterpret_cast<const ulonglong2*>(p.mA + base + k);
+                ulonglong2 e = ld_pair(p.E + base + k);
+                ulonglong2 ma = ld_pair(p.mA + base + k);
                 ulonglong2 w = *reinterpret_cast<const ulonglong2*>(p.vmb + k);
                 ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p.vf + k);
                 acc += e.x * w.x + e.y * w.y;
@@ -544,10 +548,10 @@ __global__ void __launch_bounds__(NT) rows_group_kernel(const __grid_constant__ 
     const int64_t task = ((int64_t)blockIdx.x - g.rb[li]) * WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (L.rp.fold) {
-        if (W == 1 && L.rows_vec2) rows_body<W, 2, true>(L.rp, task, lane);
+        if (W == 1 && L.rows_vec2) rows_body<W, 2, true, true>(L.rp, task, lane);
         else rows_body<W, 1, true>(L.rp, task, lane);
     } else {
-        if (W == 1 && L.rows_vec2) rows_body<W, 2, false>(L.rp, task, lane);
+        if (W == 1 && L.rows_vec2) rows_body<W, 2, false, true>(L.rp, task, lane);
         else rows_body<W, 1, false>(L.rp, task, lane);
     }
 }
