@@ -90,6 +90,11 @@ __device__ __forceinline__ ulonglong2 ld_pair(const u64* p) {
     asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
     return v;
 }
+__device__ __forceinline__ u64 ld_word(const u64* p) {
+    u64 v;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
 // streaming (evict-first) 16-byte load / store for data read or written once
 __device__ __forceinline__ ulonglong2 ld_stream2(const u64* p) {
     ulonglong2 v;
