@@ -54,6 +54,9 @@ __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const
     using T = typename Elem<W>::T;
     constexpr int U = 4;
     const int blocks = CLUSTER ? CHECK_CLUSTER : 1, rank = CLUSTER ? (int)ptx::cluster_rank() : 0;
+    // 300,000 rows with the loads held in place or left to the compiler: Z_2^64 14.5
+    // or 11.3 us, Z_2^128 19.1 or 24.8
+    auto row = [](const u64* p, int64_t i) { return W == 2 ? ld_here<W>(p, i) : ld_elem<W>(p, i); };
     const T a = ld_elem<W>(alpha, 0);
     T acc = 0;
     const int64_t step = (int64_t)blocks * NT;
@@ -62,9 +65,9 @@ __device__ __forceinline__ void check_compact(int64_t M, const u64* alpha, const
         T x[U], d[U], m[U];
 #pragma unroll
         for (int i = 0; i < U; ++i) {
-            x[i] = ld_elem<W>(chi_hat, r + i * step);
-            d[i] = ld_elem<W>(Dc, r + i * step);
-            m[i] = ld_elem<W>(mDc, r + i * step);
+            x[i] = row(chi_hat, r + i * step);
+            d[i] = row(Dc, r + i * step);
+            m[i] = row(mDc, r + i * step);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) acc += x[i] * (a * d[i] - m[i]);
@@ -131,13 +134,13 @@ __device__ __forceinline__ void sweep(int64_t n, const u64* Wm, const u64* mW, F
         T w[U], m[U];
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-            w[j] = ld_elem<W>(Wm, i + j * step);
-            m[j] = ld_elem<W>(mW, i + j * step);
+            w[j] = ld_here<W>(Wm, i + j * step);
+            m[j] = ld_here<W>(mW, i + j * step);
         }
 #pragma unroll
         for (int j = 0; j < U; ++j) f(i + j * step, w[j], m[j]);
     }
-    for (; i < n; i += step) f(i, ld_elem<W>(Wm, i), ld_elem<W>(mW, i));
+    for (; i < n; i += step) f(i, ld_here<W>(Wm, i), ld_here<W>(mW, i));
 }
 
 template <int W>
@@ -147,10 +150,10 @@ __global__ void __launch_bounds__(NT) batchrec_partial_kernel(int64_t n, const u
     ptx::grid_dep_launch();
     ptx::grid_dep_wait();   // launched as a dependent of the kernel before it
     using T = typename Elem<W>::T;
-    const T a = ld_elem<W>(alpha, 0);
+    const T a = ld_here<W>(alpha, 0);
     T acc = 0;
     sweep<W>(n, Wm, mW, [&](int64_t i, T w, T m) {
-        const T x = ld_elem<W>(chi, i);
+        const T x = ld_here<W>(chi, i);
         acc += m * x - a * (w * x);
     });
     T tot = block_sum<W>(acc);

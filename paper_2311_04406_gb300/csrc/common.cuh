@@ -95,6 +95,15 @@ __device__ __forceinline__ u64 ld_word(const u64* p) {
     asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
     return v;
 }
+template <int W>
+__device__ __forceinline__ typename Elem<W>::T ld_here(const u64* p, int64_t i) {
+    if constexpr (W == 1) {
+        return ld_word(p + i);
+    } else {
+        const ulonglong2 v = ld_pair(p + 2 * i);
+        return (u128)v.x | ((u128)v.y << 64);
+    }
+}
 // streaming (evict-first) 16-byte load / store for data read or written once
 __device__ __forceinline__ ulonglong2 ld_stream2(const u64* p) {
     ulonglong2 v;
