@@ -68,7 +68,7 @@ size_t gemm_ws(const mpc_layer* L, bool least, int one_half = 0) {
 
 // Whether the residue path runs the layer in this workspace.  If it was chosen but
 // the workspace is too small or not 256-byte aligned, c becomes the choice among
-// the other paths, which judge the workspace by their own needs (the integer pipes
+// the other paths, which hold the workspace to their own needs (the integer pipes
 // have none).
 bool use_crt(mpcl::Choice& c, const mpcl::GemmArgs& g, const void* ws, size_t ws_bytes) {
     if (!c.crt) return false;

@@ -23,7 +23,7 @@ def lib():
 
 
 @pytest.mark.hidden_gpu
-def test_workspace_is_judged_by_the_path_that_runs(lib):
+def test_workspace_is_held_to_the_path_that_runs(lib):
     L = abi.make_layer(*ODD)
     need = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE)
     assert abi.mpc_launch_count(L, abi.MPC_WS_SHARE) == 3 and need > 0
@@ -35,7 +35,7 @@ def test_workspace_is_judged_by_the_path_that_runs(lib):
     # also when a table entry names the path
     abi.mpc_autotune_set(L, 1, tile_rows=256)
     assert share(0x10010) == abi.MPC_E_CUDA and share(None) == abi.MPC_E_CUDA
-    # the digit tiles judge the workspace as ever
+    # the digit tiles hold the workspace to their needs as ever
     L = abi.make_layer(64, 256, 256)
     digits = abi.mpc_workspace_size(L, abi.MPC_WS_SHARE)
     abi.mpc_autotune_set(L, 1, tile_rows=256)
